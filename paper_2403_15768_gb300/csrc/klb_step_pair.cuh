@@ -127,22 +127,35 @@ __device__ __forceinline__ void moments2(const float2 g[Q], float2 &m, float2 j[
     }
 }
 
-// Pull direction i of both cells.  SHIFT is the x shift of the direction's
-// source (+1: from x - 1, -1: from x + 1, 0: none).
-template <typename S, bool REF>
-__device__ __forceinline__ float2 pull_dir(const S *__restrict__ in, int src, int shift, const Cols &X,
-                                           float ref, float inv)
+// Pull the Q populations of both cells.  A direction with c_x = 0 comes
+// from one aligned pair; one with c_x != 0 from two scalars, at x - c_x or,
+// on the rows where an x-moving population bounces back (XB: its bit is in
+// neither shift mask), at x itself.  The columns are selected, not branched
+// on: with a branch per direction the 16-bit decode sat inside it and every
+// load of such a row was waited for before the next was issued.
+template <int Q, typename S, bool XB>
+__device__ __forceinline__ void pull_cols(const S *__restrict__ in, const int src[Q], uint32_t moves,
+                                          const Cols &X, const float *dec, float inv, float2 g[Q])
 {
-    const S *q = src_row(in, src);
-    float2 v;
-    if (shift == 0)
-        v = Pair<S>::load2(q + X.x0);
-    else if (shift > 0)
-        v = make_float2(Pair<S>::load1(q + X.pm_a), Pair<S>::load1(q + X.x0));
-    else
-        v = make_float2(Pair<S>::load1(q + X.pp_a), Pair<S>::load1(q + X.pp_b));
-    if constexpr (REF) v = fma2(v, b2(inv), b2(ref));
-    return v;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        const S *q = src_row(in, src[i]);
+        if (cx<Q>(i) == 0) {
+            g[i] = Pair<S>::load2(q + X.x0);
+            continue;
+        }
+        int a = cx<Q>(i) > 0 ? X.pm_a : X.pp_a, b = cx<Q>(i) > 0 ? X.x0 : X.pp_b;
+        if constexpr (XB) {
+            const bool still = !((moves >> i) & 1u);
+            a = still ? X.x0 : a;
+            b = still ? X.x0 + 1 : b;
+        }
+        g[i] = make_float2(Pair<S>::load1(q + a), Pair<S>::load1(q + b));
+    }
+    if constexpr (Storage<S>::kRef) {
+#pragma unroll
+        for (int i = 0; i < Q; ++i) g[i] = fma2(g[i], b2(inv), b2(__ldg(dec + i)));
+    }
 }
 
 template <int Q, typename S>
@@ -150,18 +163,10 @@ __device__ __forceinline__ void pull_row2(const S *__restrict__ in, const int sr
                                           uint32_t xp, bool xbounce, const Cols &X, const float *dec,
                                           float inv, float2 g[Q])
 {
-    constexpr bool REF = Storage<S>::kRef;
-    if (!xbounce) {
-#pragma unroll
-        for (int i = 0; i < Q; ++i)
-            g[i] = pull_dir<S, REF>(in, src[i], cx<Q>(i), X, REF ? __ldg(dec + i) : 0.f, inv);
-    } else {
-#pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            const int sh = ((xm >> i) & 1u) ? 1 : (((xp >> i) & 1u) ? -1 : 0);
-            g[i] = pull_dir<S, REF>(in, src[i], sh, X, REF ? __ldg(dec + i) : 0.f, inv);
-        }
-    }
+    if (!xbounce)
+        pull_cols<Q, S, false>(in, src, 0u, X, dec, inv, g);
+    else
+        pull_cols<Q, S, true>(in, src, xm | xp, X, dec, inv, g);
 }
 
 __device__ __forceinline__ float2 ld2(const float *p) { return *reinterpret_cast<const float2 *>(p); }
@@ -174,7 +179,11 @@ __device__ __forceinline__ float2 lagged2(const float *U1, const float *U2, int 
 __device__ __forceinline__ float2 rcp2(float2 r) { return make_float2(1.f / r.x, 1.f / r.y); }
 
 // Uw1, Uw2 / Us1, Us2: the lagged velocities of the two steps before the
-// time level of g (water / solid), as in water_math.
+// time level of g (water / solid), as in water_math.  The faces are the outer
+// loop and the components unrolled inside it, so that a face's velocities (6
+// or 12 loads) are in flight together: with the components outside, each of
+// the 3 x (1 + faces) groups was waited for in turn, and those rows, a tenth
+// of a pipe, set a small lattice's step time.
 template <int Q>
 __device__ __forceinline__ void water_math2(const StepArgs<float> &p, const float *Uw1, const float *Uw2,
                                             const float *Us1, const float *Us2, const RowInfo &R, int x0,
@@ -188,17 +197,24 @@ __device__ __forceinline__ void water_math2(const StepArgs<float> &p, const floa
     if (slot >= 0) {
         const int ns_w = p.n_slots[kFluid], ns_s = p.n_slots[kSolid], nxp = p.nxp;
         const int nface = R.nface;
+        float2 uw[3], f[3];
+#pragma unroll
         for (int a = 0; a < 3; ++a) {
-            const float2 uw = lagged2(Uw1, Uw2, (a * ns_w + slot) * nxp + x0);
-            float2 f = b2(0.f);
-            for (int k = 0; k < nface; ++k) {
-                const int q = R.partner[k];
-                const float2 de = sub2(uw, lagged2(Us1, Us2, (a * ns_s + q) * nxp + x0));
-                const float2 dp = sub2(uw, lagged2(Us1, Us2, ((a + 3) * ns_s + q) * nxp + x0));
-                f = sub2(f, fma2(b2(p.g_we), de, mul2(b2(p.g_wp), dp)));
-            }
-            c.F[a] = add2(c.F[a], f);
+            uw[a] = lagged2(Uw1, Uw2, (a * ns_w + slot) * nxp + x0);
+            f[a] = b2(0.f);
         }
+#pragma unroll 1
+        for (int k = 0; k < nface; ++k) {
+            const int q = R.partner[k];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const float2 de = sub2(uw[a], lagged2(Us1, Us2, (a * ns_s + q) * nxp + x0));
+                const float2 dp = sub2(uw[a], lagged2(Us1, Us2, ((a + 3) * ns_s + q) * nxp + x0));
+                f[a] = sub2(f[a], fma2(b2(p.g_we), de, mul2(b2(p.g_wp), dp)));
+            }
+        }
+#pragma unroll
+        for (int a = 0; a < 3; ++a) c.F[a] = add2(c.F[a], f[a]);
     }
     const float2 rinv = rcp2(add2(b2(p.rho0), c.drho));
 #pragma unroll
@@ -218,17 +234,20 @@ __device__ __forceinline__ void solid_math2(const StepArgs<float> &p, const floa
     if (slot >= 0) {
         const int ns_w = p.n_slots[kFluid], ns_s = p.n_slots[kSolid], nxp = p.nxp;
         const int nface = R.nface;
+        float2 ue[3], up[3];
+#pragma unroll
         for (int a = 0; a < 3; ++a) {
-            const float2 ue = lagged2(Us1, Us2, (a * ns_s + slot) * nxp + x0);
-            const float2 up = lagged2(Us1, Us2, ((a + 3) * ns_s + slot) * nxp + x0);
-            float2 fe = b2(0.f), fp = b2(0.f);
-            for (int k = 0; k < nface; ++k) {
+            ue[a] = lagged2(Us1, Us2, (a * ns_s + slot) * nxp + x0);
+            up[a] = lagged2(Us1, Us2, ((a + 3) * ns_s + slot) * nxp + x0);
+        }
+#pragma unroll 1
+        for (int k = 0; k < nface; ++k) {
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
                 const float2 uw = lagged2(Uw1, Uw2, (a * ns_w + R.partner[k]) * nxp + x0);
-                fe = fma2(b2(p.g_we), sub2(uw, ue), fe);
-                fp = fma2(b2(p.g_wp), sub2(uw, up), fp);
+                Fe[a] = fma2(b2(p.g_we), sub2(uw, ue[a]), Fe[a]);
+                Fp[a] = fma2(b2(p.g_wp), sub2(uw, up[a]), Fp[a]);
             }
-            Fe[a] = fe;
-            Fp[a] = fp;
         }
     }
     // (a + k + se) ue - k up = Je,  -k ue + (b + k + sp) up = Jp.
