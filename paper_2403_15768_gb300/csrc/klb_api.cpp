@@ -81,10 +81,17 @@ void *dev(const klb_lattice *L, size_t off) { return L->base + off; }
 // Lagged-velocity slot of step m (slots rotate with period 3).
 int slot_of(int64_t m) { return (int)(((m % 3) + 3) % 3); }
 
+// Bytes of a lattice's two state buffers.
+size_t state_bytes(const klb_lattice *L)
+{
+    return 2 * (L->plan.pop_bytes[0] + L->plan.pop_bytes[1] + L->plan.pop_bytes[2]);
+}
+
 // Kernel arguments for the time level `st` (the step about to run, or the
-// one observed); the step kernel runs blocks of sbx threads.
+// one observed); the step kernel runs blocks of sbx threads and touches
+// all_bytes of state buffers per launch.
 template <typename T>
-void fill_args_at(const klb_lattice *L, const HostState &st, int sbx, StepArgs<T> &a)
+void fill_args_at(const klb_lattice *L, const HostState &st, int sbx, size_t all_bytes, StepArgs<T> &a)
 {
     const Geometry &g = L->geo;
     const MemoryPlan &p = L->plan;
@@ -147,12 +154,13 @@ void fill_args_at(const klb_lattice *L, const HostState &st, int sbx, StepArgs<T
     a.step_lo = (uint32_t)((uint64_t)n & 0xffffffffu);
     a.step_hi = (uint32_t)((uint64_t)n >> 32);
     a.bounds_err = (unsigned *)dev(L, p.bounds);
+    a.ahead = step_ahead(g.Q, d.storage, g.nxp, all_bytes);
 }
 
 template <typename T>
 void fill_args(const klb_lattice *L, StepArgs<T> &a)
 {
-    fill_args_at(L, L->st, L->plan.sbx, a);
+    fill_args_at(L, L->st, L->plan.sbx, state_bytes(L), a);
 }
 
 // The host side of one step: encode generation of the output, whether the
@@ -916,6 +924,8 @@ klb_status build_tables(klb_batch *B, int width)
     std::vector<int> prefix(n + 1, 0);
     B->plans.assign((size_t)P * n, StepPlan{0, false, false});
     B->acc.assign(P, 0);
+    size_t all_bytes = 0;
+    for (const klb_lattice *L : B->mem) all_bytes += state_bytes(L);
     for (int m = 0; m < n; ++m) {
         const klb_lattice *L = B->mem[m];
         HostState st = L->st;
@@ -927,13 +937,13 @@ klb_status build_tables(klb_batch *B, int width)
             const uint32_t *reps = (const uint32_t *)(B->base + B->reps_off);
             if (B->storage == KLB_FP64) {
                 StepArgs<double> a;
-                fill_args_at(L, st, width, a);
+                fill_args_at(L, st, width, all_bytes, a);
                 a.step_reps = reps;
                 a.step_period = P;
                 std::memcpy(slot, &a, sizeof a);
             } else {
                 StepArgs<float> a;
-                fill_args_at(L, st, width, a);
+                fill_args_at(L, st, width, all_bytes, a);
                 a.step_reps = reps;
                 a.step_period = P;
                 if (reduced(L))

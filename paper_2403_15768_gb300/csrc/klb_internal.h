@@ -132,6 +132,23 @@ inline size_t storage_bytes(int storage)
     return storage == KLB_FP64 ? 8 : (storage == KLB_FP32 ? 4 : 2);
 }
 
+// Distance, in rows, of the step's L2 requests (prefetch_rows); 0: none.
+// They pay once the state buffers (all_bytes, of every lattice in the launch)
+// exceed the 129 MB L2, so that the populations have left it by the next
+// step: step times without -> with, GB300, FP32 at 108 MB 17.4 -> 18.6 us,
+// 162 MB 33.1 -> 32.4, 270 MB 51.3 -> 47.7, 865 MB 134.9 -> 130.4, 2.9 GB
+// 437.8 -> 428.2; FP16 at 108 MB 32.2 -> 32.2, 135 MB 47.9 -> 46.7, 433 MB
+// 114.8 -> 109.3, 1.5 GB 366.6 -> 347.0.  FP32 is best at 2 MB of populations
+// (4 MB: 131.8 us at 865 MB, 10 MB: 141.7), 16 bits at 4 MB (2 MB: 355.0 us
+// at 1.5 GB, 10 MB: 352.8).
+constexpr size_t kL2Bytes = 129000000;
+inline int step_ahead(int Q, int storage, int nxp, size_t all_bytes)
+{
+    if (storage == KLB_FP64 || all_bytes <= kL2Bytes) return 0;
+    const size_t ahead = reduced_storage(storage) ? 4u << 20 : 2u << 20, row = (size_t)Q * nxp * storage_bytes(storage);
+    return (int)((ahead + row - 1) / row);
+}
+
 // Kernel arguments.  T is the arithmetic type (float or double); the
 // populations are stored as T, or as FP16/BF16 against per-row references.
 template <typename T>
@@ -166,6 +183,7 @@ struct alignas(16) StepArgs {
     // periods completed since the tables were built (null for one lattice)
     const uint32_t *step_reps;
     int step_period;
+    int ahead;             // rows ahead whose populations the step asks L2 for (step_ahead; 0: none)
     unsigned *bounds_err;  // debug builds: first out-of-range index site
 };
 

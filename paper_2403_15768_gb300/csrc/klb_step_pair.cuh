@@ -455,6 +455,38 @@ __device__ __forceinline__ int thread_segment(const StepArgs<float> &p, bool wat
     return (water ? 0 : p.nseg_w) + row * p.nch32 + xs / 32;
 }
 
+// Ask L2 for populations that later blocks will read: the same chunk of the
+// row p.ahead rows on (the water rows follow the solid rows), so that their
+// loads find them on the chip.  The registers let a warp have one item's
+// loads outstanding and no more, which for 16-bit populations (half the
+// bytes per load) left HBM half idle and for FP32 a few percent.  The rows
+// are asked for as they lie, [direction][row][x], not as they are pulled: a
+// row's sources are its neighbours, asked for by the blocks around it.  One
+// thread per direction, one bulk request each; blocks of 32 or 64 threads
+// leave it to every fourth or second chunk of a row, for as many chunks at
+// once.  See step_ahead for the distance.
+template <int Q, typename S>
+__device__ __forceinline__ void prefetch_rows(const StepArgs<float> &p, bool water, int row, int ch)
+{
+    const int G = blockDim.x <= 32 ? 4 : (blockDim.x <= 64 ? 2 : 1);
+    int r = row + p.ahead;
+    if (!water && r >= p.n_rows[kSolid]) {
+        r -= p.n_rows[kSolid];
+        water = true;
+    }
+    const int nr = p.n_rows[water ? kFluid : kSolid];
+    if ((int)threadIdx.x >= Q || (ch & (G - 1)) || r >= nr) return;
+    const int xs = ch * 2 * (int)blockDim.x;
+    const uint32_t bytes = (uint32_t)min(2 * G * (int)blockDim.x, p.nxp - xs) * (uint32_t)sizeof(S);
+    const long long off = ((long long)(int)threadIdx.x * nr + r) * p.nxp + xs;
+    const S *q = static_cast<const S *>(p.in[water ? 0 : 1]) + off;
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(q), "r"(bytes) : "memory");
+    if (!water) {
+        q = static_cast<const S *>(p.in[2]) + off;
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(q), "r"(bytes) : "memory");
+    }
+}
+
 template <int Q, typename S, bool ACC, bool NOISE = false>
 __device__ __forceinline__ void step_body2(const StepArgs<float> &p, int b)
 {
@@ -465,6 +497,9 @@ __device__ __forceinline__ void step_body2(const StepArgs<float> &p, int b)
     const int bb = water ? b - nsb : b;
     const int nch = water ? p.snchunk_w : p.snchunk_s;
     int row = bb / nch;
+    if constexpr (!NOISE) {
+        if (p.ahead) prefetch_rows<Q, S>(p, water, row, bb - row * nch);
+    }
     const int xt = (bb - row * nch) * blockDim.x + threadIdx.x;
     const int x_first = 2 * xt;
     bool live = x_first < p.nx;
