@@ -288,15 +288,15 @@ klb_status klb_observables(klb_lattice *lat, klb_obs *out);
  * Same inputs and output as klb_observables() (the lattice state is read, the
  * observables are written to *out on the host).  The per-block FP64 partial
  * sums and the final sums live in a static device array of this library
- * instead of the lattice buffer: KLB_STATIC_MAX_BLOCKS blocks of 19 doubles
- * plus 32 doubles (about 7.5 MB), held on every GPU that loads the library
+ * instead of the lattice buffer: KLB_STATIC_MAX_BLOCKS blocks of 15 doubles
+ * plus 32 doubles (about 5.9 MB), held on every GPU that loads the library
  * until the process exits.  Nothing is allocated: no cudaMalloc, cudaFree or
  * allocating library routine is called.
  *
- * - Lattices whose observation pass needs more than KLB_STATIC_MAX_BLOCKS
- *   thread blocks (per cross-section cell, one per 256 x positions with
- *   FP32 arithmetic, one per 128 with FP64 storage) are rejected with
- *   KLB_EINVAL and a message naming the limit.
+ * - Lattices of more than KLB_STATIC_MAX_BLOCKS row chunks (per
+ *   cross-section cell, one per 256 x positions with FP32 arithmetic, one per
+ *   128 with FP64 storage) are rejected with KLB_EINVAL and a message naming
+ *   the limit.
  * - The first call on a device looks up the device address of the array
  *   (once per device, with that device current); make that first call before
  *   any stream capture.

@@ -227,11 +227,35 @@ cudaError_t refresh_refs(const klb_lattice *L, int gen)
 
 int nblocks(const klb_lattice *L) { return L->plan.nblocks_w + L->plan.nblocks_s; }
 
-// Grid of the observation pass: with FP32 arithmetic two cells per thread on
-// the step kernel's grid (at most nblocks(L) blocks, the size of the partial
-// sums region), with FP64 one cell per thread.
-int obs_blocks(const klb_lattice *L) { return L->desc.storage == KLB_FP64 ? nblocks(L) : L->plan.snblocks; }
-int obs_bx(const klb_lattice *L) { return L->desc.storage == KLB_FP64 ? L->plan.bx : L->plan.sbx; }
+// Observation pass enqueued on the lattice's stream, its kNumSums sums in
+// `sums`: one kernel with FP32 arithmetic (`done` counts its finished
+// blocks, 0 before and after), the pass and its final reduction with FP64.
+cudaError_t launch_observe(const klb_lattice *L, double *partials, double *sums, unsigned *done)
+{
+    if (L->desc.storage == KLB_FP64) {
+        StepArgs<double> a;
+        fill_args(L, a);
+        a.partials = partials;
+        cudaError_t e = launch(L->geo.Q, L->desc.storage, &a, kModeObserve, nblocks(L), L->plan.bx, L->stream);
+        return e != cudaSuccess ? e : launch_finalize(partials, nblocks(L), sums, L->stream);
+    }
+    StepArgs<float> a;
+    fill_args(L, a);
+    a.partials = partials;
+    a.obs_sums = sums;
+    a.obs_done = done;
+    a.obs_solid = L->plan.oblocks_s;
+    return launch(L->geo.Q, L->desc.storage, &a, kModeObserve, L->plan.oblocks, kBlockX, L->stream);
+}
+
+cudaError_t launch_observe(const klb_lattice *L)
+{
+    return launch_observe(L, (double *)dev(L, L->plan.partials), (double *)dev(L, L->plan.sums),
+                          (unsigned *)dev(L, L->plan.obs_done));
+}
+
+// Blocks that bound the lattices klb_observables_static takes.
+int static_blocks(const klb_lattice *L) { return L->desc.storage == KLB_FP64 ? nblocks(L) : L->plan.snblocks; }
 
 // Species field index helpers: row class and row count of species s.
 int cls_of(int s) { return s == 0 ? kFluid : kSolid; }
@@ -322,7 +346,7 @@ klb_status finish_observables(klb_lattice *L, const double *S, klb_obs *out)
     out->step = L->st.step;
     out->flow_rate = S[kSumUxFluid] / g.nx;
     out->d_wall = g.has_fit ? g.d_wall : nan;
-    const double n = S[kSumFitN], s2 = S[kSumFitD2], s4 = S[kSumFitD4];
+    const double n = g.fit_n, s2 = g.fit_d2, s4 = g.fit_d4;
     const double su = S[kSumFitU], su2 = S[kSumFitUD2];
     const double det = n * s4 - s2 * s2;
     if (g.has_fit && n >= 2 && det != 0.0) {
@@ -335,7 +359,7 @@ klb_status finish_observables(klb_lattice *L, const double *S, klb_obs *out)
     } else {
         out->fit_A = out->fit_B = out->u_slip = out->dudn_wall = out->slip_length = nan;
     }
-    out->u_wallrow_mean = S[kSumWallN] > 0 ? S[kSumWallU] / S[kSumWallN] : nan;
+    out->u_wallrow_mean = g.wall_n > 0 ? S[kSumWallU] / g.wall_n : nan;
     const double ncells[3] = {(double)g.rows[kFluid].size() * g.nx,
                               (double)g.rows[kSolid].size() * g.nx,
                               (double)g.rows[kSolid].size() * g.nx};
@@ -432,6 +456,7 @@ klb_status klb_create_lattice(const klb_desc *desc, void *dev_buf, size_t bytes,
                             sizeof(RowInfo) * L->geo.info[c].size(), cudaMemcpyHostToDevice,
                             L->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(dev(L, L->plan.bounds), 0, sizeof(unsigned), L->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(dev(L, L->plan.obs_done), 0, sizeof(unsigned), L->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(L->stream);
     if (e != cudaSuccess) {
         std::string m = std::string("uploading row tables: ") + cudaGetErrorString(e);
@@ -529,12 +554,7 @@ klb_status klb_step(klb_lattice *L, int64_t nsteps)
 // synchronise the shared stream once, then finish each from its sums.
 cudaError_t klb::observe_enqueue(klb_lattice *L, double *host_sums)
 {
-    cudaError_t e = with_args(L, [&](void *a) {
-        return launch(L->geo.Q, L->desc.storage, a, kModeObserve, obs_blocks(L), obs_bx(L), L->stream);
-    });
-    if (e == cudaSuccess)
-        e = launch_finalize((const double *)dev(L, L->plan.partials), obs_blocks(L), (double *)dev(L, L->plan.sums),
-                            L->stream);
+    cudaError_t e = launch_observe(L);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(host_sums, dev(L, L->plan.sums), sizeof(double) * kNumSums, cudaMemcpyDeviceToHost,
                             L->stream);
@@ -551,12 +571,7 @@ extern "C" {
 klb_status klb_observables(klb_lattice *L, klb_obs *out)
 {
     if (!L || !out) return fail(L, KLB_EINVAL, "null argument");
-    KLB_CUDA(L, with_args(L, [&](void *a) {
-                 return launch(L->geo.Q, L->desc.storage, a, kModeObserve, obs_blocks(L),
-                                    obs_bx(L), L->stream);
-             }));
-    KLB_CUDA(L, launch_finalize((const double *)dev(L, L->plan.partials), obs_blocks(L),
-                                (double *)dev(L, L->plan.sums), L->stream));
+    KLB_CUDA(L, launch_observe(L));
     double S[kNumSums];
     KLB_CUDA(L, cudaMemcpyAsync(S, dev(L, L->plan.sums), sizeof S, cudaMemcpyDeviceToHost,
                                 L->stream));
@@ -571,20 +586,12 @@ klb_status klb_observables_static(klb_lattice *L, klb_obs *out)
     double *partials = nullptr, *sums = nullptr;
     size_t max_blocks = 0;
     KLB_CUDA(L, static_scratch(&partials, &sums, &max_blocks));
-    if ((size_t)obs_blocks(L) > max_blocks)
+    if ((size_t)static_blocks(L) > max_blocks)
         return fail(L, KLB_EINVAL,
-                    "observation pass needs " + std::to_string(obs_blocks(L)) +
+                    "observation pass needs " + std::to_string(static_blocks(L)) +
                         " blocks, more than the static scratch holds (KLB_STATIC_MAX_BLOCKS = " +
                         std::to_string(max_blocks) + ")");
-    KLB_CUDA(L, with_args(L, [&](void *a) {
-                 if (L->desc.storage == KLB_FP64)
-                     static_cast<StepArgs<double> *>(a)->partials = partials;
-                 else
-                     static_cast<StepArgs<float> *>(a)->partials = partials;
-                 return launch(L->geo.Q, L->desc.storage, a, kModeObserve, obs_blocks(L),
-                                    obs_bx(L), L->stream);
-             }));
-    KLB_CUDA(L, launch_finalize(partials, obs_blocks(L), sums, L->stream));
+    KLB_CUDA(L, launch_observe(L, partials, sums, reinterpret_cast<unsigned *>(sums + kNumSums)));
     double S[kNumSums];
     KLB_CUDA(L, cudaMemcpyAsync(S, sums, sizeof S, cudaMemcpyDeviceToHost, L->stream));
     klb_status st = sync(L);

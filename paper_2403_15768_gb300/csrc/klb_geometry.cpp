@@ -296,6 +296,12 @@ bool build_geometry(const klb_desc &d, Geometry &g, std::string &err)
         ri.d2 = (float)(dist * dist);
         if (g.has_fit && (g.d_wall - dist) >= 4.0) ri.flags |= kFitRow;
         if (ri.nface > 0) ri.flags |= kWallRow;
+        if (ri.flags & kFitRow) {
+            g.fit_n += d.nx;
+            g.fit_d2 += d.nx * (double)ri.d2;
+            g.fit_d4 += d.nx * ((double)ri.d2 * (double)ri.d2);
+        }
+        if (ri.flags & kWallRow) g.wall_n += d.nx;
     }
     return true;
 }
@@ -333,8 +339,20 @@ MemoryPlan plan_memory(const Geometry &g, int storage)
         p.snblocks = (int)nr[kFluid] * step_chunks(g.nx, p.sbx, storage, true) +
                      (int)nr[kSolid] * step_chunks(g.nx, p.sbx, storage, false);
     }
-    p.partials = take(sizeof(double) * kNumSums * (size_t)(p.nblocks_w + p.nblocks_s));
-    p.sums = take(sizeof(double) * kNumSums);
+    {
+        // Observation grid: at most the 4 blocks of 4 warps that fit an SM at
+        // 128 registers, no more blocks than items (64 cells of a row) need,
+        // split between the classes by work (a solid item pulls two species).
+        const int nseg = (g.nx + 63) / 64, wpb = kBlockX / 32;
+        const double is = (double)nr[kSolid] * nseg, iw = (double)nr[kFluid] * nseg;
+        const int ms = (int)std::min(1e9, std::ceil(is / wpb)), mw = (int)std::min(1e9, std::ceil(iw / wpb));
+        const int total = (int)std::min((double)kObsBlocks, (double)ms + mw);
+        p.oblocks_s = std::min(ms, std::max(1, (int)std::lround(total * 2 * is / (2 * is + iw))));
+        p.oblocks = p.oblocks_s + std::min(mw, std::max(1, total - p.oblocks_s));
+    }
+    p.partials = take(sizeof(double) * kNumSums * std::max((size_t)(p.nblocks_w + p.nblocks_s), (size_t)p.oblocks));
+    p.sums = take(sizeof(double) * kNumSums + sizeof(unsigned));
+    p.obs_done = p.sums + sizeof(double) * kNumSums;
     p.field_bytes = ts * 4 * (nr[kFluid] + 2 * nr[kSolid]) * g.nxp;
     p.field = take(p.field_bytes);
     for (int s = 0; s < 3; ++s) p.ref_bytes[s] = 0;

@@ -14,6 +14,7 @@ namespace klb {
 
 constexpr int kMaxFaces = 4;   // fluid/solid faces of one cross-section cell (+-y, +-z)
 constexpr int kBlockX = 128;   // threads per block along x (one x per thread)
+constexpr int kObsBlocks = 4 * 152;  // resident blocks of the observation pass (FP32 arithmetic)
 // Rows are padded to a multiple of kRowAlign elements.  RowInfo::src counts
 // in these units, so a 32-bit entry reaches 2^31 * 32 elements of a class
 // buffer; offsets within one direction plane (row * nxp + x) stay 32-bit.
@@ -42,16 +43,12 @@ static_assert(sizeof(RowInfo) == 128, "RowInfo is one 128-byte line");
 
 enum RowFlags { kFitRow = 1, kWallRow = 2, kXBounce = 4 };
 
-// Indices of the FP64 partial sums reduced by the observation kernel.
+// Indices of the FP64 sums of the observation pass.
 enum SumIndex {
     kSumUxFluid = 0,   // sum of u_x over fluid cells
-    kSumFitN,          // slip fit: count, sum d^2, sum d^4, sum u, sum u d^2
-    kSumFitD2,
-    kSumFitD4,
-    kSumFitU,
+    kSumFitU,          // sum of u_x and of u_x d^2 over the slip fit's cells
     kSumFitUD2,
-    kSumWallN,         // wall-row count and sum u_x
-    kSumWallU,
+    kSumWallU,         // sum of u_x over the wall rows
     kSumUxE,           // electron / phonon sum u_x
     kSumUxP,
     kSumMomW,          // sum rho u_x per species
@@ -78,6 +75,7 @@ struct Geometry {
     int max_faces[2] = {0, 0};
     double d_wall = 0.0;
     bool has_fit = false;
+    double fit_n = 0, fit_d2 = 0, fit_d4 = 0, wall_n = 0;  // cells of the slip fit with sums of d^2, d^4; wall-row cells
 };
 
 // Builds the geometry and its streaming / interface tables.  Returns false
@@ -91,7 +89,7 @@ struct MemoryPlan {
     size_t U[3][2];        // [time slot][row class]
     size_t U_bytes[2];
     size_t rows[2];
-    size_t partials, sums, field;
+    size_t partials, sums, obs_done, field;
     size_t field_bytes;
     size_t ref_enc[2][3], ref_dec[2][3];  // [generation][species], reduced storage only
     size_t ref_bytes[3];
@@ -100,6 +98,7 @@ struct MemoryPlan {
     size_t total;
     int nblocks_w, nblocks_s, nchunk, bx;  // one cell per thread (observe, field, init)
     int sbx, snblocks;                     // step kernel: threads per block, blocks
+    int oblocks, oblocks_s;                // observation with FP32 arithmetic: blocks of kBlockX, of which solid
 };
 MemoryPlan plan_memory(const Geometry &g, int storage);
 
@@ -167,6 +166,9 @@ struct alignas(16) StepArgs {
     T g_we, g_wp, g_ep, g_ec, g_pc;
     T q_p;                 // phonons: 1 second-order equilibrium, 0 linear (damped waves, Sec. 3.4)
     double *partials;      // observe mode: [block][kNumSums]
+    double *obs_sums;      // observe mode, FP32 arithmetic: the final sums,
+    unsigned *obs_done;    // blocks done (0 between passes)
+    int obs_solid;         // and blocks that take the solid rows
     int residual_valid;
     T *field;              // field / init mode: per species [4][n_rows][nxp]
     // reduced-precision storage only (null otherwise)
@@ -203,6 +205,7 @@ cudaError_t launch(int Q, int storage, const void *args, int mode, int nblocks, 
 // Reference refresh from args.acc into the tables enc[s], dec[s].
 cudaError_t launch_ref(int Q, int storage, const void *args, float *const enc[3],
                        float *const dec[3], cudaStream_t s);
+// Final sums of the FP64 observation pass (with FP32 arithmetic the pass writes them itself).
 cudaError_t launch_finalize(const double *partials, int nblocks, double *sums, cudaStream_t s);
 // One more period completed by a batch (StepArgs::step_reps).
 cudaError_t launch_count_period(uint32_t *reps, cudaStream_t s);

@@ -41,7 +41,7 @@ cudaError_t launch_ref(int Q, int storage, const void *args, float *const enc[3]
 // reduces sum k.  Each thread keeps four accumulators over interleaved
 // partials (four independent loads in flight), combines them in a fixed
 // order, then the block reduces the threads' values in a fixed tree.
-constexpr int kFinalizeThreads = 1024;
+constexpr int kFinalizeThreads = 256;
 
 __global__ void __launch_bounds__(kFinalizeThreads) k_finalize(const double *__restrict__ partials, int nblocks,
                                                                double *__restrict__ sums)

@@ -102,7 +102,7 @@ template <> struct Storage<double> {
 };
 // 16-bit encodes round to nearest and saturate: a value beyond the largest
 // finite magnitude is stored as that magnitude (not as infinity), which the
-// observation pass counts (clipped_cell); NaN stays NaN.
+// observation pass counts (clipped2); NaN stays NaN.
 __device__ __forceinline__ unsigned short f32_to_f16_sat(float v)
 {
     unsigned short r;
@@ -131,7 +131,7 @@ __device__ __forceinline__ unsigned f32x2_to_bf16x2_sat(float2 v)
 
 template <> struct Storage<__half> {
     static constexpr bool kRef = true;
-    static constexpr unsigned short kMaxBits = 0x7bffu;  // 65504
+    static constexpr float kMax = 65504.f;  // largest finite magnitude
     __device__ static float load(const __half *p)
     {
         return __half2float(__ushort_as_half(__ldg(reinterpret_cast<const unsigned short *>(p))));
@@ -143,7 +143,7 @@ template <> struct Storage<__half> {
 };
 template <> struct Storage<__nv_bfloat16> {
     static constexpr bool kRef = true;
-    static constexpr unsigned short kMaxBits = 0x7f7fu;  // 3.3895e38
+    static constexpr float kMax = 3.38953139e38f;  // largest finite magnitude, (2 - 2^-7) 2^127
     __device__ static float load(const __nv_bfloat16 *p)
     {
         return __bfloat162float(
@@ -154,26 +154,6 @@ template <> struct Storage<__nv_bfloat16> {
         *reinterpret_cast<unsigned short *>(p) = f32_to_bf16_sat(v);
     }
 };
-
-// Whether any of the Q pulled 16-bit populations of a cell sits at the
-// largest finite magnitude (a saturated encode); false for wider storage.
-template <int Q, typename S>
-__device__ __forceinline__ bool clipped_cell(const S *__restrict__ in, const RowInfo &R, int x, int xm1, int xp1)
-{
-    if constexpr (!Storage<S>::kRef) {
-        return false;
-    } else {
-        bool any = false;
-#pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            const int xs = ((R.xm >> i) & 1u) ? xm1 : (((R.xp >> i) & 1u) ? xp1 : x);
-            const unsigned short b =
-                __ldg(reinterpret_cast<const unsigned short *>(in + (long long)R.src[i] * kRowAlign + xs));
-            any |= (b & 0x7fffu) == Storage<S>::kMaxBits;
-        }
-        return any;
-    }
-}
 
 // ---------------------------------------------------------------------------
 
@@ -512,17 +492,15 @@ __device__ __forceinline__ double warp_max(double v)
     return v;
 }
 
-// Block sums of the observation pass (one row chunk per block, so the row
-// class and flags are block-uniform; ncell = the thread's live cells).  Only the sums that can be non-zero
-// for the block's class run a warp reduction (FP64 throughput on GB300 is a
-// small fraction of FP32); the slip-fit count and distance moments and the wall-row count
-// follow from the number of live cells and the row's d^2, the fit and
-// wall-row u_x sums are the u_x sum itself (every cell of such a row adds
-// its u_x to both), and non-finite values are counted with block-wide
-// predicate counts.  Each entry equals what a reduction of the per-cell
-// values gives.
-__device__ inline void observe_reduce_store(const double (&s)[kNumSums], bool water, int flags, double d2,
-                                            int ncell, double *out)
+// Block sums of the FP64 observation pass (one cell per thread, one row chunk
+// per block, so the row class and flags are block-uniform).  Only the sums
+// that can be non-zero for the block's class run a warp reduction (FP64
+// throughput on GB300 is a small fraction of FP32); the fit and wall-row u_x
+// sums are the u_x sum itself (every cell of such a row adds its u_x to
+// both), non-finite values are counted with block-wide predicate counts, and
+// the counts and distance moments of the slip fit come from the geometry on
+// the host.
+__device__ inline void observe_reduce_store(const double (&s)[kNumSums], bool water, int flags, double *out)
 {
     __shared__ double red[kNumSums][kBlockX / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -533,14 +511,7 @@ __device__ inline void observe_reduce_store(const double (&s)[kNumSums], bool wa
                     (fit ? (1u << kSumFitUD2) : 0u)
               : (1u << kSumUxE) | (1u << kSumUxP) | (1u << kSumMomE) | (1u << kSumMomP) | (1u << kSumMassE) |
                     (1u << kSumMassP) | (1u << kSumResidual);
-    const int cnt = __syncthreads_count(ncell >= 1) + __syncthreads_count(ncell >= 2);  // live cells
-    // per-thread counts of up to four species-cells (two cells of two species)
-    auto count4 = [](double v) {
-        return __syncthreads_count(v >= 1.0) + __syncthreads_count(v >= 2.0) + __syncthreads_count(v >= 3.0) +
-               __syncthreads_count(v >= 4.0);
-    };
-    const int nonfinite = count4(s[kSumNonfinite]);
-    const int clipped = count4(s[kSumClipped]);
+    const int nonfinite = __syncthreads_count(s[kSumNonfinite] >= 1.0) + __syncthreads_count(s[kSumNonfinite] >= 2.0);
 #pragma unroll
     for (int k = 0; k < kNumSums; ++k) {
         if (!((sel >> k) & 1u)) continue;
@@ -558,22 +529,12 @@ __device__ inline void observe_reduce_store(const double (&s)[kNumSums], bool wa
         double v = 0.0;
         if ((sel >> k) & 1u)
             v = total(k);
-        else if (k == kSumFitN)
-            v = fit ? (double)cnt : 0.0;
-        else if (k == kSumFitD2)
-            v = fit ? cnt * d2 : 0.0;
-        else if (k == kSumFitD4)
-            v = fit ? cnt * (d2 * d2) : 0.0;
         else if (k == kSumFitU)
             v = fit ? total(kSumUxFluid) : 0.0;
-        else if (k == kSumWallN)
-            v = wall ? (double)cnt : 0.0;
         else if (k == kSumWallU)
             v = wall ? total(kSumUxFluid) : 0.0;
         else if (k == kSumNonfinite)
             v = (double)nonfinite;
-        else if (k == kSumClipped)
-            v = (double)clipped;
         out[k] = v;
     }
 }
@@ -656,19 +617,7 @@ __global__ void __launch_bounds__(kBlockX, (sizeof(T) == 4 ? 8 : 1)) k_lattice(c
                 s[kSumMomW] = rho * ux;
                 s[kSumMassW] = (double)c.drho;
                 s[kSumNonfinite] = finite3(c) ? 0.0 : 1.0;
-                s[kSumClipped] = clipped_cell<Q, S>(static_cast<const S *>(p.in[0]), R, x, xm1, xp1) ? 1.0 : 0.0;
-                if (R.flags & kFitRow) {
-                    const double d2 = (double)R.d2;
-                    s[kSumFitN] = 1.0;
-                    s[kSumFitD2] = d2;
-                    s[kSumFitD4] = d2 * d2;
-                    s[kSumFitU] = ux;
-                    s[kSumFitUD2] = ux * d2;
-                }
-                if (R.flags & kWallRow) {
-                    s[kSumWallN] = 1.0;
-                    s[kSumWallU] = ux;
-                }
+                if (R.flags & kFitRow) s[kSumFitUD2] = ux * (double)R.d2;
                 if (p.residual_valid) {
                     Cell<T> cprev;
                     pull<Q, T, S>(static_cast<const S *>(p.in_prev[0]), R, x, xm1, xp1,
@@ -707,8 +656,6 @@ __global__ void __launch_bounds__(kBlockX, (sizeof(T) == 4 ? 8 : 1)) k_lattice(c
                 s[kSumMassE] = (double)ce.drho;
                 s[kSumMassP] = (double)cp.drho;
                 s[kSumNonfinite] = (finite3(ce) ? 0.0 : 1.0) + (finite3(cp) ? 0.0 : 1.0);
-                s[kSumClipped] = (clipped_cell<Q, S>(static_cast<const S *>(p.in[1]), R, x, xm1, xp1) ? 1.0 : 0.0) +
-                                 (clipped_cell<Q, S>(static_cast<const S *>(p.in[2]), R, x, xm1, xp1) ? 1.0 : 0.0);
                 if (p.residual_valid) {
                     Cell<T> pe, pp;
                     pull<Q, T, S>(static_cast<const S *>(p.in_prev[1]), R, x, xm1, xp1,
@@ -724,8 +671,7 @@ __global__ void __launch_bounds__(kBlockX, (sizeof(T) == 4 ? 8 : 1)) k_lattice(c
     }
     if (MODE == kModeObserve) {
         const RowInfo &Rb = p.rows[water ? kFluid : kSolid][row];
-        observe_reduce_store(s, water, water ? Rb.flags : 0, (double)Rb.d2, live ? 1 : 0,
-                             p.partials + (size_t)b * kNumSums);
+        observe_reduce_store(s, water, water ? Rb.flags : 0, p.partials + (size_t)b * kNumSums);
     }
 }
 
@@ -1227,8 +1173,8 @@ cudaError_t launch_q(const void *args, int mode, int nblocks, int bx, cudaStream
         else
             return cudaErrorInvalidValue;
     case kModeObserve:
-        // FP32 arithmetic: two cells per thread on the step grid (the caller
-        // passes its blocks and width); FP64: one cell per thread
+        // FP32 arithmetic: two cells per thread on a resident grid; FP64:
+        // one cell per thread (the caller passes blocks and width)
         if constexpr (sizeof(T) == 4)
             k_observe2<Q, S><<<nblocks, bx, 0, s>>>(a);
         else

@@ -133,9 +133,10 @@ __device__ __forceinline__ void moments2(const float2 g[Q], float2 &m, float2 j[
 // neither shift mask), at x itself.  The columns are selected, not branched
 // on: with a branch per direction the 16-bit decode sat inside it and every
 // load of such a row was waited for before the next was issued.
-template <int Q, typename S, bool XB>
+// CLIP (16-bit storage): top takes the largest stored magnitude of each cell.
+template <int Q, typename S, bool XB, bool CLIP>
 __device__ __forceinline__ void pull_cols(const S *__restrict__ in, const int src[Q], uint32_t moves,
-                                          const Cols &X, const float *dec, float inv, float2 g[Q])
+                                          const Cols &X, const float *dec, float inv, float2 g[Q], float2 &top)
 {
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
@@ -154,19 +155,24 @@ __device__ __forceinline__ void pull_cols(const S *__restrict__ in, const int sr
     }
     if constexpr (Storage<S>::kRef) {
 #pragma unroll
-        for (int i = 0; i < Q; ++i) g[i] = fma2(g[i], b2(inv), b2(__ldg(dec + i)));
+        for (int i = 0; i < Q; ++i) {
+            if constexpr (CLIP) top = make_float2(fmaxf(top.x, fabsf(g[i].x)), fmaxf(top.y, fabsf(g[i].y)));
+            g[i] = fma2(g[i], b2(inv), b2(__ldg(dec + i)));
+        }
     }
 }
 
-template <int Q, typename S>
+template <int Q, typename S, bool CLIP = false>
 __device__ __forceinline__ void pull_row2(const S *__restrict__ in, const int src[Q], uint32_t xm,
                                           uint32_t xp, bool xbounce, const Cols &X, const float *dec,
-                                          float inv, float2 g[Q])
+                                          float inv, float2 g[Q], float2 *top = nullptr)
 {
+    float2 t = make_float2(0.f, 0.f);
     if (!xbounce)
-        pull_cols<Q, S, false>(in, src, 0u, X, dec, inv, g);
+        pull_cols<Q, S, false, CLIP>(in, src, 0u, X, dec, inv, g, t);
     else
-        pull_cols<Q, S, true>(in, src, xm | xp, X, dec, inv, g);
+        pull_cols<Q, S, true, CLIP>(in, src, xm | xp, X, dec, inv, g, t);
+    if constexpr (CLIP) *top = t;
 }
 
 __device__ __forceinline__ float2 ld2(const float *p) { return *reinterpret_cast<const float2 *>(p); }
@@ -609,11 +615,26 @@ __device__ __forceinline__ void step_body2(const StepArgs<float> &p, int b)
     }
 }
 
-// Observation pass with two cells per thread (FP32 arithmetic), on the step
-// kernel's grid (solid blocks first): the velocities of the current step
-// (lagged velocities U1, U2) and, for the residual, of the previous one (U2,
-// U3), from the same pulls and arithmetic as the step, reduced per block in
-// FP64 into the partial sums of the observation (observe_reduce_store).
+// Observation pass with two cells per thread (FP32 arithmetic): the
+// velocities of the current step (lagged velocities U1, U2) and, for the
+// residual, of the previous one (U2, U3), from the same pulls and arithmetic
+// as the step, summed in FP64.
+//
+// What bounds it: the two states (2 x 19 populations per species-cell) and
+// the FP64 pipe, 2 lanes per clock and SM.  A resident grid walks the items
+// (64 cells of a row, one per warp and turn; the solid items on the first
+// obs_solid blocks, the water items on the others, in proportion to their
+// work), so that each thread keeps its sums in registers and the FP64
+// reductions over threads run once per block instead of once per row chunk;
+// the residual's FP64 difference is formed only for cells that can raise the
+// maximum.  The last block to finish sums the blocks' partials in block
+// order (the same order every time).  Counts and distance moments of the
+// slip fit are properties of the geometry and computed on the host.
+// klb_observables, GB300, before (a block per row chunk, FP64 sums and a
+// reduction kernel over them) -> now: 512x128x128 FP32 388 -> 192 us, FP16
+// 463 -> 189; 768x192x192 FP32 1214 -> 535, FP16 1460 -> 511; 128x64x64 FP32
+// 55 -> 45; pipe R8 nx 8 43 -> 31.  L2 requests for the next item, as in the
+// step, were slower (239 us): two states stream through L2 here.
 __device__ __forceinline__ bool finite2(const Cell2 &c, int e)
 {
     const float v[4] = {e ? c.drho.y : c.drho.x, e ? c.u[0].y : c.u[0].x, e ? c.u[1].y : c.u[1].x,
@@ -621,35 +642,72 @@ __device__ __forceinline__ bool finite2(const Cell2 &c, int e)
     return isfinite(v[0]) && isfinite(v[1]) && isfinite(v[2]) && isfinite(v[3]);
 }
 
+// Running maximum of |a - b| in FP64: the FP32 difference decides whether
+// the exact one can exceed it (its rounding is within 2^-24).
+struct MaxDiff {
+    double m = 0.0;
+    float lim = 0.f;
+    __device__ __forceinline__ void add(float a, float b)
+    {
+        if (fabsf(a - b) >= lim) {
+            const double e = fabs((double)a - (double)b);
+            if (e > m) {
+                m = e;
+                lim = (float)e * 0.999999f;
+            }
+        }
+    }
+};
+
+// Cells of a pair whose largest stored magnitude is the largest finite one
+// (the encode saturates, so nothing larger is stored; NaN does not count).
+template <typename S>
+__device__ __forceinline__ int clipped2(float2 top, bool both)
+{
+    const float m = Storage<S>::kMax;
+    return (top.x == m ? 1 : 0) + (both && top.y == m ? 1 : 0);
+}
+
+// Values of a block's partial row: six sums (water: u_x, momentum, mass, u_x
+// and u_x d^2 of the fit rows, u_x of the wall rows; solid: u_x, momentum,
+// mass of electrons and phonons in turn), residual, non-finite and clipped
+// species-cells.
+constexpr int kObsValues = 9;
+
 template <int Q, typename S>
 __global__ void __launch_bounds__(kBlockX, 4) k_observe2(const StepArgs<float> p)
 {
-    const int b = blockIdx.x;
-    const int nsb = p.n_rows[kSolid] * p.snchunk_s;
-    const bool water = b >= nsb;
-    const int bb = water ? b - nsb : b;
-    const int nch = water ? p.snchunk_w : p.snchunk_s;
-    int row = bb / nch;
-    const int x_first = 2 * ((bb - row * nch) * (int)blockDim.x + (int)threadIdx.x);
-    bool live = x_first < p.nx;
-    if constexpr (KLB_BOUNDS) {
-        if (live && !row_indices_ok<Q>(p, water, row, 0, x_first + 1)) {
-            live = false;
-            row = 0;
+    constexpr bool kRef = Storage<S>::kRef;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool water = (int)blockIdx.x >= p.obs_solid;
+    const int cls = water ? kFluid : kSolid;
+    const int nb = water ? (int)gridDim.x - p.obs_solid : p.obs_solid;
+    const int wpb = blockDim.x >> 5, nseg = (p.nx + 63) / 64;
+    const int items = p.n_rows[cls] * nseg;
+    double s[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    MaxDiff res;
+    int nonfinite = 0, clipped = 0;
+    for (int it = ((int)blockIdx.x - (water ? p.obs_solid : 0)) * wpb + warp; it < items; it += nb * wpb) {
+        // a warp's row, in a uniform register (a warp-wide reduction of equal
+        // values tells the compiler so: the row record then needs no vector ones)
+        int row = (int)__reduce_max_sync(0xffffffffu, (unsigned)(it / nseg));
+        const int x_first = (it - row * nseg) * 64 + 2 * lane;
+        bool live = x_first < p.nx;
+        if constexpr (KLB_BOUNDS) {
+            const bool ok = !live || row_indices_ok<Q>(p, water, row, 0, x_first + 1);
+            if (!__all_sync(0xffffffffu, ok)) {
+                live = false;
+                row = 0;
+            }
         }
-    }
-    const bool both = live && x_first + 1 < p.nx;
-    double s[kNumSums];
-#pragma unroll
-    for (int k = 0; k < kNumSums; ++k) s[k] = 0.0;
-    const RowInfo &R = p.rows[water ? kFluid : kSolid][row];
-    if (live) {
+        const bool both = live && x_first + 1 < p.nx;
         Cols X;
-        X.x0 = x_first;
+        X.x0 = live ? x_first : 0;
         X.pm_a = X.x0 == 0 ? p.nx - 1 : X.x0 - 1;
         X.pp_a = X.x0 + 1 >= p.nx ? 0 : X.x0 + 1;
         X.pp_b = X.x0 + 2 >= p.nx ? 0 : X.x0 + 2;
         const float inv = p.inv_scale;
+        const RowInfo &R = p.rows[cls][row];
         const int4 *t4 = reinterpret_cast<const int4 *>(&R);
         int src[20];
 #pragma unroll
@@ -666,7 +724,8 @@ __global__ void __launch_bounds__(kBlockX, 4) k_observe2(const StepArgs<float> p
         const uint32_t xp = (uint32_t)q5.x;
         const bool xbounce = (q7.x & kXBounce) != 0;
         // the previous step first (for the residual), keeping only its u_x,
-        // so that the current step's values and sums are live alone
+        // so that the current step's values are live alone; the second cell
+        // of an odd row's last pair lies in the padding and enters no sum
         if (water) {
             float2 g[Q], j[3];
             float2 uq = b2(0.f);
@@ -678,22 +737,31 @@ __global__ void __launch_bounds__(kBlockX, 4) k_observe2(const StepArgs<float> p
                 uq = cq.u[0];
             }
             Cell2 c;
-            pull_row2<Q, S>(static_cast<const S *>(p.in[0]), src, xm, xp, xbounce, X,
-                            ref_row<float, S>(p.dec_in[0], row), inv, g);
-            water_math2<Q>(p, p.U1[kFluid], p.U2[kFluid], p.U1[kSolid], p.U2[kSolid], R, X.x0, g, c, j);
-            const double u0 = c.u[0].x, u1 = both ? (double)c.u[0].y : 0.0;
-            s[kSumUxFluid] = u0 + u1;
-            // the second cell of an odd row's last pair lies in the padding:
-            // none of its values enters a sum
-            s[kSumMomW] = (double)(p.rho0 + c.drho.x) * u0 + (both ? (double)(p.rho0 + c.drho.y) * u1 : 0.0);
-            s[kSumMassW] = (double)c.drho.x + (both ? (double)c.drho.y : 0.0);
-            s[kSumNonfinite] = (finite2(c, 0) ? 0.0 : 1.0) + (both && !finite2(c, 1) ? 1.0 : 0.0);
             const S *in0 = static_cast<const S *>(p.in[0]);
-            s[kSumClipped] = (clipped_cell<Q, S>(in0, R, X.x0, X.pm_a, X.pp_a) ? 1.0 : 0.0) +
-                             (both && clipped_cell<Q, S>(in0, R, X.x0 + 1, X.x0, X.pp_b) ? 1.0 : 0.0);
-            if (R.flags & kFitRow) s[kSumFitUD2] = (u0 + u1) * (double)R.d2;
-            if (p.residual_valid)
-                s[kSumResidual] = fmax(fabs(u0 - (double)uq.x), both ? fabs(u1 - (double)uq.y) : 0.0);
+            float2 top;
+            pull_row2<Q, S, kRef>(in0, src, xm, xp, xbounce, X, ref_row<float, S>(p.dec_in[0], row), inv, g, &top);
+            water_math2<Q>(p, p.U1[kFluid], p.U2[kFluid], p.U1[kSolid], p.U2[kSolid], R, X.x0, g, c, j);
+            if (live) {
+                const double u0 = c.u[0].x, u1 = both ? (double)c.u[0].y : 0.0, uu = u0 + u1;
+                s[0] += uu;
+                s[1] = fma((double)(p.rho0 + c.drho.x), u0, s[1]);
+                s[2] += (double)c.drho.x;
+                if (both) {
+                    s[1] = fma((double)(p.rho0 + c.drho.y), u1, s[1]);
+                    s[2] += (double)c.drho.y;
+                }
+                if (q7.x & kFitRow) {
+                    s[3] += uu;
+                    s[4] = fma(uu, (double)R.d2, s[4]);
+                }
+                if (q7.x & kWallRow) s[5] += uu;
+                nonfinite += (finite2(c, 0) ? 0 : 1) + (both && !finite2(c, 1) ? 1 : 0);
+                if constexpr (kRef) clipped += clipped2<S>(top, both);
+                if (p.residual_valid) {
+                    res.add(c.u[0].x, uq.x);
+                    if (both) res.add(c.u[0].y, uq.y);
+                }
+            }
         } else {
             float2 ge[Q], gp[Q], je[3], jp[3];
             float2 eq = b2(0.f), pq = b2(0.f);
@@ -709,36 +777,117 @@ __global__ void __launch_bounds__(kBlockX, 4) k_observe2(const StepArgs<float> p
                 pq = qp.u[0];
             }
             Cell2 ce, cp;
-            pull_row2<Q, S>(static_cast<const S *>(p.in[1]), src, xm, xp, xbounce, X,
-                            ref_row<float, S>(p.dec_in[1], row), inv, ge);
-            pull_row2<Q, S>(static_cast<const S *>(p.in[2]), src, xm, xp, xbounce, X,
-                            ref_row<float, S>(p.dec_in[2], row), inv, gp);
+            const S *in1 = static_cast<const S *>(p.in[1]), *in2 = static_cast<const S *>(p.in[2]);
+            float2 te, tp;
+            pull_row2<Q, S, kRef>(in1, src, xm, xp, xbounce, X, ref_row<float, S>(p.dec_in[1], row), inv, ge, &te);
+            pull_row2<Q, S, kRef>(in2, src, xm, xp, xbounce, X, ref_row<float, S>(p.dec_in[2], row), inv, gp, &tp);
             solid_math2<Q>(p, p.U1[kFluid], p.U2[kFluid], p.U1[kSolid], p.U2[kSolid], R, X.x0, ge, gp, ce, cp, je,
                            jp);
-            const double e0 = ce.u[0].x, e1 = both ? (double)ce.u[0].y : 0.0;
-            const double p0 = cp.u[0].x, p1 = both ? (double)cp.u[0].y : 0.0;
-            s[kSumUxE] = e0 + e1;
-            s[kSumUxP] = p0 + p1;
-            s[kSumMomE] = (double)(p.rho0 + ce.drho.x) * e0 + (both ? (double)(p.rho0 + ce.drho.y) * e1 : 0.0);
-            s[kSumMomP] = (double)(p.rho0 + cp.drho.x) * p0 + (both ? (double)(p.rho0 + cp.drho.y) * p1 : 0.0);
-            s[kSumMassE] = (double)ce.drho.x + (both ? (double)ce.drho.y : 0.0);
-            s[kSumMassP] = (double)cp.drho.x + (both ? (double)cp.drho.y : 0.0);
-            s[kSumNonfinite] = (finite2(ce, 0) ? 0.0 : 1.0) + (finite2(cp, 0) ? 0.0 : 1.0) +
-                               (both && !finite2(ce, 1) ? 1.0 : 0.0) + (both && !finite2(cp, 1) ? 1.0 : 0.0);
-            const S *in1 = static_cast<const S *>(p.in[1]), *in2 = static_cast<const S *>(p.in[2]);
-            s[kSumClipped] = (clipped_cell<Q, S>(in1, R, X.x0, X.pm_a, X.pp_a) ? 1.0 : 0.0) +
-                             (clipped_cell<Q, S>(in2, R, X.x0, X.pm_a, X.pp_a) ? 1.0 : 0.0) +
-                             (both && clipped_cell<Q, S>(in1, R, X.x0 + 1, X.x0, X.pp_b) ? 1.0 : 0.0) +
-                             (both && clipped_cell<Q, S>(in2, R, X.x0 + 1, X.x0, X.pp_b) ? 1.0 : 0.0);
-            if (p.residual_valid) {
-                double r = fmax(fabs(e0 - (double)eq.x), fabs(p0 - (double)pq.x));
-                if (both) r = fmax(r, fmax(fabs(e1 - (double)eq.y), fabs(p1 - (double)pq.y)));
-                s[kSumResidual] = r;
+            if (live) {
+                auto add = [&](const Cell2 &c, double &su, double &sm, double &sd) {
+                    const double u0 = c.u[0].x;
+                    su += u0;
+                    sm = fma((double)(p.rho0 + c.drho.x), u0, sm);
+                    sd += (double)c.drho.x;
+                    if (both) {
+                        const double u1 = c.u[0].y;
+                        su += u1;
+                        sm = fma((double)(p.rho0 + c.drho.y), u1, sm);
+                        sd += (double)c.drho.y;
+                    }
+                    nonfinite += (finite2(c, 0) ? 0 : 1) + (both && !finite2(c, 1) ? 1 : 0);
+                };
+                add(ce, s[0], s[1], s[2]);
+                add(cp, s[3], s[4], s[5]);
+                if constexpr (kRef) clipped += clipped2<S>(te, both) + clipped2<S>(tp, both);
+                if (p.residual_valid) {
+                    res.add(ce.u[0].x, eq.x);
+                    res.add(cp.u[0].x, pq.x);
+                    if (both) {
+                        res.add(ce.u[0].y, eq.y);
+                        res.add(cp.u[0].y, pq.y);
+                    }
+                }
             }
         }
     }
-    observe_reduce_store(s, water, water ? R.flags : 0, (double)R.d2, live ? (both ? 2 : 1) : 0,
-                         p.partials + (size_t)b * kNumSums);
+
+    // the block's partial row
+    __shared__ double red[kBlockX / 32][kObsValues];
+    __shared__ bool last;
+    nonfinite = __reduce_add_sync(0xffffffffu, nonfinite);
+    clipped = __reduce_add_sync(0xffffffffu, clipped);
+    const double rm = warp_max(res.m);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        const double v = warp_sum(s[k]);
+        if (lane == 0) red[warp][k] = v;
+    }
+    if (lane == 0) {
+        red[warp][6] = rm;
+        red[warp][7] = (double)nonfinite;
+        red[warp][8] = (double)clipped;
+    }
+    __syncthreads();
+    if (threadIdx.x < kObsValues) {
+        const int k = threadIdx.x;
+        double v = red[0][k];
+        for (int w = 1; w < wpb; ++w) v = k == 6 ? fmax(v, red[w][k]) : v + red[w][k];
+        p.partials[(size_t)blockIdx.x * kNumSums + k] = v;
+        __threadfence();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(p.obs_done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    // the last block: warp 0 the solid blocks, the next (or the same) the water blocks
+    __threadfence();
+    if (threadIdx.x < kNumSums) p.obs_sums[threadIdx.x] = 0.0;
+    __syncthreads();
+    double *shared_res = &red[0][0];
+    for (int c = warp; c < 2; c += wpb) {
+        const int b0 = c == 0 ? 0 : p.obs_solid, b1 = c == 0 ? p.obs_solid : (int)gridDim.x;
+        double t[kObsValues];
+#pragma unroll
+        for (int k = 0; k < kObsValues; ++k) t[k] = 0.0;
+#pragma unroll 4
+        for (int b = b0 + lane; b < b1; b += 32) {
+            const double *q = p.partials + (size_t)b * kNumSums;
+#pragma unroll
+            for (int k = 0; k < kObsValues; ++k) {
+                const double v = __ldcg(q + k);
+                t[k] = k == 6 ? fmax(t[k], v) : t[k] + v;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < kObsValues; ++k) t[k] = k == 6 ? warp_max(t[k]) : warp_sum(t[k]);
+        if (lane == 0) {
+            double *o = p.obs_sums;
+            if (c == 0) {
+                o[kSumUxE] = t[0];
+                o[kSumMomE] = t[1];
+                o[kSumMassE] = t[2];
+                o[kSumUxP] = t[3];
+                o[kSumMomP] = t[4];
+                o[kSumMassP] = t[5];
+            } else {
+                o[kSumUxFluid] = t[0];
+                o[kSumMomW] = t[1];
+                o[kSumMassW] = t[2];
+                o[kSumFitU] = t[3];
+                o[kSumFitUD2] = t[4];
+                o[kSumWallU] = t[5];
+            }
+            for (int k = 0; k < 3; ++k) shared_res[c * 3 + k] = t[6 + k];
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        p.obs_sums[kSumResidual] = fmax(shared_res[0], shared_res[3]);
+        p.obs_sums[kSumNonfinite] = shared_res[1] + shared_res[4];
+        p.obs_sums[kSumClipped] = shared_res[2] + shared_res[5];
+        *p.obs_done = 0u;  // for the next observation (stream order)
+    }
 }
 
 }  // namespace klb
