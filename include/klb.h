@@ -364,12 +364,12 @@ klb_status klb_batch_create(klb_lattice *const *members, int n, void *dev_buf, s
 klb_status klb_batch_step(klb_batch *b, int64_t nsteps);
 
 /* Time steps_per_candidate >= 1 steps of the batch with each block width
- * (32, 64 and 128 consecutive x per thread block) and keep the fastest; the
+ * (32, 64 and 128 threads) and keep the fastest; the
  * timed steps are real steps of the members.  *width (may be NULL) receives
  * the chosen width.  Synchronises. */
 klb_status klb_batch_autotune(klb_batch *b, int steps_per_candidate, int *width);
 
-/* Block width in use (128 unless autotuned) and total blocks per step. */
+/* Block width (threads) in use and total blocks per step. */
 int klb_batch_width(const klb_batch *b);
 int64_t klb_batch_blocks(const klb_batch *b);
 

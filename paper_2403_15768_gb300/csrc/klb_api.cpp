@@ -127,9 +127,14 @@ void fill_args_at(const klb_lattice *L, const HostState &st, int sbx, size_t all
     a.nxp = g.nxp;
     a.nchunk = p.nchunk;
     a.nbw = (int)g.rows[kFluid].size() * a.nchunk;
-    a.snchunk_w = step_chunks(g.nx, sbx, L->desc.storage, true);
-    a.snchunk_s = step_chunks(g.nx, sbx, L->desc.storage, false);
-    a.snbw = (int)g.rows[kFluid].size() * a.snchunk_w;
+    a.snchunk = (g.nx + sbx - 1) / sbx;
+    a.nseg64 = (g.nx + 63) / 64;
+    {
+        uint32_t sh = 0;  // division by multiplication: the kernel's first instructions wait for it
+        while ((1u << sh) < (uint32_t)a.nseg64) ++sh;
+        a.seg_shift = 31 + sh;
+        a.seg_mul = (uint32_t)((1ull << (31 + sh)) / (uint32_t)a.nseg64 + 1);
+    }
     a.nch32 = (g.nx + 31) / 32;
     a.nseg_w = (int)g.rows[kFluid].size() * a.nch32;
     const klb_desc &d = L->desc;
@@ -255,7 +260,7 @@ cudaError_t launch_observe(const klb_lattice *L)
 }
 
 // Blocks that bound the lattices klb_observables_static takes.
-int static_blocks(const klb_lattice *L) { return L->desc.storage == KLB_FP64 ? nblocks(L) : L->plan.snblocks; }
+int static_blocks(const klb_lattice *L) { return L->desc.storage == KLB_FP64 ? nblocks(L) : L->plan.static_blocks; }
 
 // Species field index helpers: row class and row count of species s.
 int cls_of(int s) { return s == 0 ? kFluid : kSolid; }
@@ -960,9 +965,8 @@ klb_status build_tables(klb_batch *B, int width)
             advance(st, sp);
         }
         const int sto = L->desc.storage;
-        prefix[m + 1] = prefix[m] +
-                        step_chunks(L->geo.nx, width, sto, true) * (int)L->geo.rows[kFluid].size() +
-                        step_chunks(L->geo.nx, width, sto, false) * (int)L->geo.rows[kSolid].size();
+        prefix[m + 1] = prefix[m] + step_blocks(L->geo.nx, (int)L->geo.rows[kFluid].size(),
+                                                (int)L->geo.rows[kSolid].size(), width, sto);
     }
     KLB_BCUDA(B, cudaStreamSynchronize(B->stream));
     KLB_BCUDA(B, cudaMemcpy(B->base + B->table_off, host.data(), host.size(), cudaMemcpyHostToDevice));
@@ -1147,7 +1151,14 @@ klb_status klb_batch_create(klb_lattice *const *members, int n, void *dev_buf, s
         return fail(nullptr, KLB_ECUDA, m);
     }
     int w = kBlockX;
-    for (klb_lattice *L : B->mem) w = std::min(w, L->plan.sbx);
+    if (B->storage == KLB_FP64) {
+        for (klb_lattice *L : B->mem) w = std::min(w, L->plan.sbx);
+    } else {
+        long long items = 0;
+        for (klb_lattice *L : B->mem)
+            items += (long long)(L->geo.rows[kFluid].size() + L->geo.rows[kSolid].size()) * ((L->geo.nx + 63) / 64);
+        w = step_width(items);
+    }
     klb_status st = build_tables(B, w);
     if (st != KLB_OK) {
         std::string m = B->err;

@@ -332,13 +332,14 @@ MemoryPlan plan_memory(const Geometry &g, int storage)
     p.nchunk = (g.nx + p.bx - 1) / p.bx;
     p.nblocks_w = (int)nr[kFluid] * p.nchunk;
     p.nblocks_s = (int)nr[kSolid] * p.nchunk;
-    {
-        const int c = step_cells(storage, false);
-        const int xt = (g.nx + c - 1) / c;  // threads per solid row
-        p.sbx = std::min(kBlockX, std::max(32, (xt + 31) / 32 * 32));
-        p.snblocks = (int)nr[kFluid] * step_chunks(g.nx, p.sbx, storage, true) +
-                     (int)nr[kSolid] * step_chunks(g.nx, p.sbx, storage, false);
+    if (storage == KLB_FP64) {
+        p.sbx = p.bx;
+        p.static_blocks = p.nblocks_w + p.nblocks_s;
+    } else {
+        p.sbx = step_width((long long)(nr[kFluid] + nr[kSolid]) * ((g.nx + 63) / 64));
+        p.static_blocks = (int)(nr[kFluid] + nr[kSolid]) * ((g.nx + 255) / 256);
     }
+    p.snblocks = step_blocks(g.nx, (int)nr[kFluid], (int)nr[kSolid], p.sbx, storage);
     {
         // Observation grid: at most the 4 blocks of 4 warps that fit an SM at
         // 128 registers, no more blocks than items (64 cells of a row) need,

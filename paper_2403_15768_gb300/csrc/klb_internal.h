@@ -98,6 +98,7 @@ struct MemoryPlan {
     size_t total;
     int nblocks_w, nblocks_s, nchunk, bx;  // one cell per thread (observe, field, init)
     int sbx, snblocks;                     // step kernel: threads per block, blocks
+    int static_blocks;                     // row chunks that klb_observables_static bounds
     int oblocks, oblocks_s;                // observation with FP32 arithmetic: blocks of kBlockX, of which solid
 };
 MemoryPlan plan_memory(const Geometry &g, int storage);
@@ -110,20 +111,20 @@ constexpr int kRefStride = 20;
 constexpr int kRefEvery = 32;
 constexpr float kFp16Scale = 1048576.0f;  // 2^20
 
-// Cells per thread of the step kernel: FP64 one; FP32 arithmetic two
-// adjacent x (packed f32x2).  Per row class, so that the classes may differ.
-inline int step_cells(int storage, bool water)
+// Blocks of sbx threads of one step launch: FP64 one block per row chunk of
+// sbx cells; FP32 arithmetic one warp per item of 64 cells (two adjacent x
+// per thread, packed f32x2).
+inline int step_blocks(int nx, int rows_w, int rows_s, int sbx, int storage)
 {
-    (void)water;
-    return storage == KLB_FP64 ? 1 : 2;
+    const long long rows = (long long)rows_w + rows_s;
+    if (storage == KLB_FP64) return (int)(rows * ((nx + sbx - 1) / sbx));
+    return (int)((rows * ((nx + 63) / 64) + sbx / 32 - 1) / (sbx / 32));
 }
 
-// Step-kernel x chunks per row of the given class for blocks of sbx threads.
-inline int step_chunks(int nx, int sbx, int storage, bool water)
-{
-    const int xb = sbx * step_cells(storage, water);
-    return (nx + xb - 1) / xb;
-}
+// Threads per step block with FP32 arithmetic: four warps, or one where the
+// launch's items fit the chip at once anyway (20 warps on each of 152 SMs),
+// which spreads them over all SMs.
+inline int step_width(long long items) { return items <= 152 * 20 ? 32 : kBlockX; }
 
 inline bool reduced_storage(int storage) { return storage == KLB_FP16_DEV || storage == KLB_BF16_DEV; }
 inline size_t storage_bytes(int storage)
@@ -159,7 +160,9 @@ struct alignas(16) StepArgs {
     const T *U1[2], *U2[2], *U3[2];  // lagged velocities u(n-1), u(n-2), u(n-3)
     T *U0[2];                        // u(n) written here (step mode)
     int nx, nxp, nchunk, nbw;        // nchunk = x chunks of blockDim.x per row; nbw = water blocks
-    int snchunk_w, snchunk_s, snbw;  // the same for the step kernel, per row class
+    int snchunk;                     // FP64 step: x chunks of blockDim.x per row
+    int nseg64;                      // 64-wide x segments per row
+    uint32_t seg_mul, seg_shift;     // n / nseg64 = n seg_mul >> seg_shift for 0 <= n < 2^31
     int nch32, nseg_w;               // 32-wide x segments per row; water segments
     int n_rows[2], n_slots[2];
     T rho0, om[3], G[3];

@@ -913,10 +913,9 @@ __device__ __forceinline__ void step_body(const StepArgs<T> &p, int b)
 {
     // solid blocks (two species each, the heavier work) first, so that the
     // grid's last wave holds the lighter water blocks
-    const int nsb = p.n_rows[kSolid] * p.snchunk_s;
+    const int nch = p.snchunk, nsb = p.n_rows[kSolid] * nch;
     const bool water = b >= nsb;
     const int bb = water ? b - nsb : b;
-    const int nch = water ? p.snchunk_w : p.snchunk_s;
     int row = bb / nch;
     int x = (bb - row * nch) * blockDim.x + threadIdx.x;
     const int x_lane = x;
@@ -1071,26 +1070,21 @@ cudaError_t launch_step(void (*kernel)(A), int nblocks, int bx, cudaStream_t s, 
     return cudaLaunchKernelEx(&cfg, kernel, a);
 }
 
-// Many lattices in one launch: the block finds its lattice as the number of
-// lattices after the first whose first block is at or before its own
-// (prefix[] is increasing), counted by all threads at once — one round of
-// independent loads instead of a chain of dependent ones — and works from a
-// shared-memory copy of that lattice's arguments.
+// Many lattices in one launch: each warp finds its block's lattice as the
+// number of lattices after the first whose first block is at or before the
+// block (prefix[] is increasing), counted by its lanes at once (one round of
+// independent loads, no block barrier: the latency is before everything
+// else), and the block works from a shared-memory copy of that lattice's
+// arguments.
 template <int Q, typename T, typename S, bool ACC>
 __global__ void __launch_bounds__(kBlockX, (step_min_blocks<T, S>()))
     k_step_batch(const StepArgs<T> *__restrict__ table, const int *__restrict__ prefix, int n)
 {
     pdl_launch_dependents();
     __shared__ StepArgs<T> sp;
-    __shared__ int s_lid;
-    if (threadIdx.x == 0) s_lid = 0;
-    __syncthreads();
     int c = 0;
-    for (int m = 1 + (int)threadIdx.x; m < n; m += blockDim.x) c += __ldg(prefix + m) <= (int)blockIdx.x;
-    c = __reduce_add_sync(0xffffffffu, c);
-    if ((threadIdx.x & 31) == 0 && c) atomicAdd(&s_lid, c);
-    __syncthreads();
-    const int lid = s_lid;
+    for (int m = 1 + ((int)threadIdx.x & 31); m < n; m += 32) c += __ldg(prefix + m) <= (int)blockIdx.x;
+    const int lid = (int)__reduce_add_sync(0xffffffffu, (unsigned)c);
     static_assert(sizeof(StepArgs<T>) % 16 == 0, "argument record in 16-byte words");
     const int4 *src = reinterpret_cast<const int4 *>(table + lid);
     int4 *dst = reinterpret_cast<int4 *>(&sp);

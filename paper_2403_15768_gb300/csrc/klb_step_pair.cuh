@@ -461,30 +461,32 @@ __device__ __forceinline__ int thread_segment(const StepArgs<float> &p, bool wat
     return (water ? 0 : p.nseg_w) + row * p.nch32 + xs / 32;
 }
 
-// Ask L2 for populations that later blocks will read: the same chunk of the
-// row p.ahead rows on (the water rows follow the solid rows), so that their
-// loads find them on the chip.  The registers let a warp have one item's
+// Ask L2 for populations that later blocks will read: the same segments of
+// the row p.ahead rows on (the water rows follow the solid rows), so that
+// their loads find them on the chip.  The registers let a warp have one item's
 // loads outstanding and no more, which for 16-bit populations (half the
 // bytes per load) left HBM half idle and for FP32 a few percent.  The rows
 // are asked for as they lie, [direction][row][x], not as they are pulled: a
-// row's sources are its neighbours, asked for by the blocks around it.  One
-// thread per direction, one bulk request each; blocks of 32 or 64 threads
-// leave it to every fourth or second chunk of a row, for as many chunks at
-// once.  See step_ahead for the distance.
+// row's sources are its neighbours, asked for by the warps around it.  Every
+// eighth segment of a row asks for eight, one lane and one bulk request per
+// direction (768x192x192 FP16: 396 us with one segment per request, 344 with
+// four, 341 with eight).  It comes first in the kernel: behind the loads of
+// the row record the step took 3% longer.  See step_ahead for the distance.
 template <int Q, typename S>
-__device__ __forceinline__ void prefetch_rows(const StepArgs<float> &p, bool water, int row, int ch)
+__device__ __forceinline__ void prefetch_rows(const StepArgs<float> &p, bool water, int row, int seg)
 {
-    const int G = blockDim.x <= 32 ? 4 : (blockDim.x <= 64 ? 2 : 1);
+    constexpr int G = 8;  // segments per request
+    const int lane = threadIdx.x & 31;
     int r = row + p.ahead;
     if (!water && r >= p.n_rows[kSolid]) {
         r -= p.n_rows[kSolid];
         water = true;
     }
     const int nr = p.n_rows[water ? kFluid : kSolid];
-    if ((int)threadIdx.x >= Q || (ch & (G - 1)) || r >= nr) return;
-    const int xs = ch * 2 * (int)blockDim.x;
-    const uint32_t bytes = (uint32_t)min(2 * G * (int)blockDim.x, p.nxp - xs) * (uint32_t)sizeof(S);
-    const long long off = ((long long)(int)threadIdx.x * nr + r) * p.nxp + xs;
+    if (lane >= Q || (seg & (G - 1)) || r >= nr) return;
+    const int xs = seg * 64;
+    const uint32_t bytes = (uint32_t)min(64 * G, p.nxp - xs) * (uint32_t)sizeof(S);
+    const long long off = ((long long)lane * nr + r) * p.nxp + xs;
     const S *q = static_cast<const S *>(p.in[water ? 0 : 1]) + off;
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(q), "r"(bytes) : "memory");
     if (!water) {
@@ -496,18 +498,26 @@ __device__ __forceinline__ void prefetch_rows(const StepArgs<float> &p, bool wat
 template <int Q, typename S, bool ACC, bool NOISE = false>
 __device__ __forceinline__ void step_body2(const StepArgs<float> &p, int b)
 {
-    // solid blocks (two species each, the heavier work) first, so that the
-    // grid's last wave holds the lighter water blocks
-    const int nsb = p.n_rows[kSolid] * p.snchunk_s;
-    const bool water = b >= nsb;
-    const int bb = water ? b - nsb : b;
-    const int nch = water ? p.snchunk_w : p.snchunk_s;
-    int row = bb / nch;
+    // An item is 64 cells of a row, one per warp; solid items (two species
+    // each, the heavier work) first, so that the grid's last wave holds the
+    // lighter water items.  Warps of a block may lie on different rows, so
+    // that narrow and ragged rows leave no warp idle; the warp-wide reduction
+    // of equal values tells the compiler that the item is warp-uniform, and
+    // the row record then stays out of the vector registers.  With a block
+    // per row chunk, one-warp blocks for narrow rows, and a division for the
+    // row: 301x77x93 slab 66.3 us (now 64.4), 193x97x97 BF16 48.0 (47.0),
+    // 12-channel sweep FP32 480.8 (475.3), FP16 457.1 (439.1).
+    const int nseg = p.nseg64, nsi = p.n_rows[kSolid] * nseg;
+    const int it = (int)__reduce_max_sync(0xffffffffu, (unsigned)(b * ((int)blockDim.x >> 5) + ((int)threadIdx.x >> 5)));
+    const bool water = it >= nsi;
+    const int ii = water ? it - nsi : it;
+    int row = (int)(((unsigned long long)(unsigned)ii * p.seg_mul) >> p.seg_shift);
+    if (water && row >= p.n_rows[kFluid]) return;
+    const int sg = ii - row * nseg;  // segment
     if constexpr (!NOISE) {
-        if (p.ahead) prefetch_rows<Q, S>(p, water, row, bb - row * nch);
+        if (p.ahead) prefetch_rows<Q, S>(p, water, row, sg);
     }
-    const int xt = (bb - row * nch) * blockDim.x + threadIdx.x;
-    const int x_first = 2 * xt;
+    const int x_first = 64 * sg + 2 * ((int)threadIdx.x & 31);
     bool live = x_first < p.nx;
     if constexpr (KLB_BOUNDS) {
         if (live && !row_indices_ok<Q>(p, water, row, 0, x_first + 1)) {
