@@ -333,13 +333,14 @@ MemoryPlan plan_memory(const Geometry &g, int storage)
     p.nblocks_w = (int)nr[kFluid] * p.nchunk;
     p.nblocks_s = (int)nr[kSolid] * p.nchunk;
     if (storage == KLB_FP64) {
-        p.sbx = p.bx;
+        p.sbx = fp64_split(g.nx, (int)nr[kFluid], (int)nr[kSolid]) ? 32 : p.bx;
         p.static_blocks = p.nblocks_w + p.nblocks_s;
     } else {
-        p.sbx = step_width((long long)(nr[kFluid] + nr[kSolid]) * ((g.nx + 63) / 64));
+        p.ep = step_ep(step_items(g.nx, nr[kFluid], nr[kSolid], true));
+        p.sbx = step_width(step_items(g.nx, nr[kFluid], nr[kSolid], p.ep));
         p.static_blocks = (int)(nr[kFluid] + nr[kSolid]) * ((g.nx + 255) / 256);
     }
-    p.snblocks = step_blocks(g.nx, (int)nr[kFluid], (int)nr[kSolid], p.sbx, storage);
+    p.snblocks = step_blocks(g.nx, (int)nr[kFluid], (int)nr[kSolid], p.sbx, storage, p.ep);
     {
         // Observation grid: at most the 4 blocks of 4 warps that fit an SM at
         // 128 registers, no more blocks than items (64 cells of a row) need,
@@ -353,6 +354,7 @@ MemoryPlan plan_memory(const Geometry &g, int storage)
     }
     p.partials = take(sizeof(double) * kNumSums * std::max((size_t)(p.nblocks_w + p.nblocks_s), (size_t)p.oblocks));
     p.sums = take(sizeof(double) * kNumSums + sizeof(unsigned));
+    p.ep = false;
     p.obs_done = p.sums + sizeof(double) * kNumSums;
     p.field_bytes = ts * 4 * (nr[kFluid] + 2 * nr[kSolid]) * g.nxp;
     p.field = take(p.field_bytes);

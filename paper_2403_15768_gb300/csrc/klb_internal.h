@@ -97,7 +97,8 @@ struct MemoryPlan {
     size_t bounds;         // error word of debug builds (KLB_BOUNDS)
     size_t total;
     int nblocks_w, nblocks_s, nchunk, bx;  // one cell per thread (observe, field, init)
-    int sbx, snblocks;                     // step kernel: threads per block, blocks
+    bool ep;                               // step kernel: form of the solid items (step_ep),
+    int sbx, snblocks;                     // threads per block, blocks
     int static_blocks;                     // row chunks that klb_observables_static bounds
     int oblocks, oblocks_s;                // observation with FP32 arithmetic: blocks of kBlockX, of which solid
 };
@@ -111,15 +112,42 @@ constexpr int kRefStride = 20;
 constexpr int kRefEvery = 32;
 constexpr float kFp16Scale = 1048576.0f;  // 2^20
 
-// Blocks of sbx threads of one step launch: FP64 one block per row chunk of
-// sbx cells; FP32 arithmetic one warp per item of 64 cells (two adjacent x
-// per thread, packed f32x2).
-inline int step_blocks(int nx, int rows_w, int rows_s, int sbx, int storage)
+// FP64 lattices of so few cells that a species-cell per thread in one-warp
+// blocks leaves SMs idle: one warp per block, and solid rows one species per
+// block.  The FP64 pipe takes 16 cycles per warp instruction on every SM, so
+// a step lasts as long as its busiest SM computes.
+inline bool fp64_split(int nx, int rows_w, int rows_s)
 {
-    const long long rows = (long long)rows_w + rows_s;
-    if (storage == KLB_FP64) return (int)(rows * ((nx + sbx - 1) / sbx));
-    return (int)((rows * ((nx + 63) / 64) + sbx / 32 - 1) / (sbx / 32));
+    return ((long long)rows_w + 2LL * rows_s) * ((nx + 31) / 32) <= 152;
 }
+
+// Blocks of sbx threads of one step launch: FP64 one block per row chunk of
+// sbx cells (a solid one per species with fp64_split); FP32 arithmetic one warp per item of 64 cells (two adjacent x
+// per thread, packed f32x2).
+inline long long step_items(int nx, long long rows_w, long long rows_s, bool ep);
+inline int step_blocks(int nx, int rows_w, int rows_s, int sbx, int storage, bool ep)
+{
+    if (storage == KLB_FP64)
+        return (rows_w + rows_s + (fp64_split(nx, rows_w, rows_s) ? rows_s : 0)) * ((nx + sbx - 1) / sbx);
+    return (int)((step_items(nx, rows_w, rows_s, ep) + sbx / 32 - 1) / (sbx / 32));
+}
+
+// Items of one launch of the FP32-arithmetic step on a lattice's rows: 64
+// cells of a row; with ep solid items are 32 cells, one per lane, electrons
+// and phonons as the pair.
+inline long long step_items(int nx, long long rows_w, long long rows_s, bool ep)
+{
+    return rows_w * ((nx + 63) / 64) + rows_s * (ep ? (nx + 31) / 32 : (nx + 63) / 64);
+}
+
+// Which form the solid items take: ep where latency counts (the items find a
+// place on the chip at about the same time): the species are pulled once, in
+// one round of loads.  Two cells and two pulls of the phonons where
+// throughput counts.  Step times with cell pairs -> with species pairs,
+// GB300, FP32: pipe R 8, nx 8 (384 items) 5.6 -> 3.8 us, nx 200 7.7 -> 5.5,
+// nx 400 (3792 items) 9.5 -> 7.7; 128x64x64 (5552 items) 8.5 -> 8.8; R 48,
+// nx 8 (9176 items) 11.0 -> 11.3; 512x128x128 134.9 -> 140.9.
+inline bool step_ep(long long ep_items) { return ep_items <= 4000; }
 
 // Threads per step block with FP32 arithmetic: four warps, or one where the
 // launch's items fit the chip at once anyway (20 warps on each of 152 SMs),
@@ -160,9 +188,11 @@ struct alignas(16) StepArgs {
     const T *U1[2], *U2[2], *U3[2];  // lagged velocities u(n-1), u(n-2), u(n-3)
     T *U0[2];                        // u(n) written here (step mode)
     int nx, nxp, nchunk, nbw;        // nchunk = x chunks of blockDim.x per row; nbw = water blocks
-    int snchunk;                     // FP64 step: x chunks of blockDim.x per row
+    int snchunk, split;              // FP64 step: x chunks of blockDim.x per row; one species per solid block
     int nseg64;                      // 64-wide x segments per row
     uint32_t seg_mul, seg_shift;     // n / nseg64 = n seg_mul >> seg_shift for 0 <= n < 2^31
+    int sseg;                        // the same for the solid rows: segments of 64, or 32 with step_ep
+    uint32_t sseg_mul, sseg_shift;
     int nch32, nseg_w;               // 32-wide x segments per row; water segments
     int n_rows[2], n_slots[2];
     T rho0, om[3], G[3];
@@ -199,7 +229,9 @@ enum Mode {
     kModeStepAcc = 3,  // step that also writes the x-sums for a refresh
     kModeInit = 4,
     kModeInitAcc = 5,  // x-sums of the initial equilibria, nothing stored
-    kModeStepNoise = 6 // step with thermal fluctuations of the water
+    kModeStepNoise = 6, // step with thermal fluctuations of the water
+    kModeStepEp = 7,    // kModeStep and kModeStepAcc with solid items of one cell per thread (step_ep)
+    kModeStepAccEp = 8
 };
 
 // Launchers (return the launch error, if any).
@@ -215,7 +247,7 @@ cudaError_t launch_count_period(uint32_t *reps, cudaStream_t s);
 // One step of many lattices in one launch: table[l] holds the arguments of
 // lattice l, prefix[l] its first block (prefix[n] = total blocks).
 cudaError_t launch_batch(int Q, int storage, const void *table, const int *prefix, int n,
-                         int nblocks, int bx, bool acc, cudaStream_t s);
+                         int nblocks, int bx, bool acc, bool ep, cudaStream_t s);
 
 // Device bytes of the argument tables of a batch of n lattices with this
 // storage (the layout klb_batch_create uses).

@@ -12,15 +12,15 @@ cudaError_t launch_ref_q9(const void *args, float *const enc[3], float *const de
 cudaError_t launch_ref_q19(const void *args, float *const enc[3], float *const dec[3], cudaStream_t s);
 
 cudaError_t launch_batch_q9(int storage, const void *table, const int *prefix, int n, int nblocks,
-                          int bx, bool acc, cudaStream_t s);
+                          int bx, bool acc, bool ep, cudaStream_t s);
 cudaError_t launch_batch_q19(int storage, const void *table, const int *prefix, int n, int nblocks,
-                           int bx, bool acc, cudaStream_t s);
+                           int bx, bool acc, bool ep, cudaStream_t s);
 
 cudaError_t launch_batch(int Q, int storage, const void *table, const int *prefix, int n,
-                         int nblocks, int bx, bool acc, cudaStream_t s)
+                         int nblocks, int bx, bool acc, bool ep, cudaStream_t s)
 {
-    return Q == 9 ? launch_batch_q9(storage, table, prefix, n, nblocks, bx, acc, s)
-                  : launch_batch_q19(storage, table, prefix, n, nblocks, bx, acc, s);
+    return Q == 9 ? launch_batch_q9(storage, table, prefix, n, nblocks, bx, acc, ep, s)
+                  : launch_batch_q19(storage, table, prefix, n, nblocks, bx, acc, ep, s);
 }
 
 cudaError_t launch(int Q, int storage, const void *args, int mode, int nblocks, int bx,

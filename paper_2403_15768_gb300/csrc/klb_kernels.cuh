@@ -254,9 +254,44 @@ __device__ __forceinline__ const float *ref_row(const float *table, int row)
 // (for u in [2^-8, 2^-7) and F = 1e-6 it is -0.48 ulp(j), -2.2e-4 F; the
 // velocity drifts by that fraction of the drive).  The remaining rounding is
 // unbiased.  g is left holding g*.
+//
+// FP64 evaluates the same terms per pair of opposite directions from sums of
+// per-axis coefficients: with T_a = om 4.5 q rho u_a + 9 q fo F_a and
+// O_a = 3 om rho u_a + 3 fo F_a (fo = 1 - om/2), om geq_i + fo F_i =
+// w_i [E + (c.u) (c.T) +- c.O].  The FP64 pipe (2 lanes per clock and SM)
+// bounds the FP64 step, and this takes 110 of its operations for D3Q19 where
+// the terms written out take 185.
+// (FP32 does not: there the roundings of separately formed axis terms add up
+// to a steady shear stress.)
 template <int Q, typename T>
 __device__ __forceinline__ void collide(T g[Q], const Cell<T> &c, const T j[3], T rho0, T om, T q = T(1))
 {
+    if constexpr (sizeof(T) == 8) {
+        const T rho = rho0 + c.drho, fo = T(1) - T(0.5) * om, om1 = T(1) - om;
+        const T uu = c.u[0] * c.u[0] + c.u[1] * c.u[1] + c.u[2] * c.u[2];
+        const T uF = c.u[0] * c.F[0] + c.u[1] * c.F[1] + c.u[2] * c.F[2];
+        const T omr = om * rho, c45 = (T(4.5) * q) * omr, c9 = (T(9) * q) * fo;
+        const T E = om * c.drho - (T(1.5) * q) * (omr * uu) - ((T(3) * q) * fo) * uF;
+        T Tv[3], O[3];
+#pragma unroll
+        for (int a = 0; a < (Q == 19 ? 3 : 2); ++a) {
+            Tv[a] = c45 * c.u[a] + c9 * c.F[a];
+            O[a] = (T(3) * omr) * c.u[a] + (T(3) * fo) * c.F[a];
+        }
+        Tv[2] = Q == 19 ? Tv[2] : T(0);
+        O[2] = Q == 19 ? O[2] : T(0);
+        g[0] = om1 * g[0] + T(wt<Q>(0)) * E;
+#pragma unroll
+        for (int i = 1; i < Q; ++i) {
+            const int ib = dir_index<Q>(-cx<Q>(i), -cy<Q>(i), -cz<Q>(i));
+            if (ib < i) continue;
+            const T w = T(wt<Q>(i));
+            const T s = E + cdot<Q, T>(i, c.u) * cdot<Q, T>(i, Tv), o = cdot<Q, T>(i, O);
+            g[i] = om1 * g[i] + w * (s + o);
+            g[ib] = om1 * g[ib] + w * (s - o);
+        }
+        return;
+    }
     const T rho = rho0 + c.drho;
     const T uu = c.u[0] * c.u[0] + c.u[1] * c.u[1] + c.u[2] * c.u[2];
     const T uF = c.u[0] * c.F[0] + c.u[1] * c.F[1] + c.u[2] * c.F[2];
@@ -370,17 +405,25 @@ __device__ __forceinline__ void water_math(const StepArgs<T> &p, const T *Uw1, c
     if (slot >= 0) {
         const int ns_w = p.n_slots[kFluid], ns_s = p.n_slots[kSolid], nxp = p.nxp;
         const int nface = R.nface;
+        // faces outside, components inside: a face's loads in flight together
+        T uw[3], f[3];
+#pragma unroll
         for (int a = 0; a < 3; ++a) {
-            const T uw = lagged(Uw1, Uw2, (a * ns_w + slot) * nxp + x);
-            T f = T(0);
-            for (int k = 0; k < nface; ++k) {
-                const int q = R.partner[k];
-                const T de = uw - lagged(Us1, Us2, (a * ns_s + q) * nxp + x);
-                const T dp = uw - lagged(Us1, Us2, ((a + 3) * ns_s + q) * nxp + x);
-                f -= p.g_we * de + p.g_wp * dp;
-            }
-            c.F[a] += f;
+            uw[a] = lagged(Uw1, Uw2, (a * ns_w + slot) * nxp + x);
+            f[a] = T(0);
         }
+#pragma unroll 1
+        for (int k = 0; k < nface; ++k) {
+            const int q = R.partner[k];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const T de = uw[a] - lagged(Us1, Us2, (a * ns_s + q) * nxp + x);
+                const T dp = uw[a] - lagged(Us1, Us2, ((a + 3) * ns_s + q) * nxp + x);
+                f[a] -= p.g_we * de + p.g_wp * dp;
+            }
+        }
+#pragma unroll
+        for (int a = 0; a < 3; ++a) c.F[a] += f[a];
     }
     const T rinv = T(1) / (p.rho0 + c.drho);
 #pragma unroll
@@ -401,17 +444,21 @@ __device__ __forceinline__ void solid_math(const StepArgs<T> &p, const T *Uw1, c
     if (slot >= 0) {
         const int ns_w = p.n_slots[kFluid], ns_s = p.n_slots[kSolid], nxp = p.nxp;
         const int nface = R.nface;
+        T ue[3], up[3];
+#pragma unroll
         for (int a = 0; a < 3; ++a) {
-            const T ue = lagged(Us1, Us2, (a * ns_s + slot) * nxp + x);
-            const T up = lagged(Us1, Us2, ((a + 3) * ns_s + slot) * nxp + x);
-            T fe = T(0), fp = T(0);
-            for (int k = 0; k < nface; ++k) {
-                const T uw = lagged(Uw1, Uw2, (a * ns_w + R.partner[k]) * nxp + x);
-                fe += p.g_we * (uw - ue);
-                fp += p.g_wp * (uw - up);
+            ue[a] = lagged(Us1, Us2, (a * ns_s + slot) * nxp + x);
+            up[a] = lagged(Us1, Us2, ((a + 3) * ns_s + slot) * nxp + x);
+        }
+#pragma unroll 1
+        for (int k = 0; k < nface; ++k) {
+            const int q = R.partner[k];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const T uw = lagged(Uw1, Uw2, (a * ns_w + q) * nxp + x);
+                Fe[a] += p.g_we * (uw - ue[a]);
+                Fp[a] += p.g_wp * (uw - up[a]);
             }
-            Fe[a] = fe;
-            Fp[a] = fp;
         }
     }
     // Trapezoidal e-p friction and sinks, solved exactly per component:
@@ -902,39 +949,38 @@ __device__ __forceinline__ void thermal_noise(const StepArgs<T> &p, uint32_t cel
     }
 }
 
-template <typename T, typename S>
+// The species-pair form (EP) runs where latency counts: 128 registers let it
+// keep more loads in flight (pipe R 24, nx 8: 4.9 us at 4 blocks, 5.5 at 5,
+// 5.9 at 3).
+template <typename T, typename S, bool EP = false>
 constexpr int step_min_blocks()
 {
-    return sizeof(T) == 8 ? 4 : 5;
+    return sizeof(T) == 8 || EP ? 4 : 5;
 }
 
-template <int Q, typename T, typename S, bool ACC, bool NOISE = false>
+// FP64: one cell per thread, one row chunk per block.
+template <int Q, typename T, typename S, bool NOISE = false>
 __device__ __forceinline__ void step_body(const StepArgs<T> &p, int b)
 {
     // solid blocks (two species each, the heavier work) first, so that the
     // grid's last wave holds the lighter water blocks
-    const int nch = p.snchunk, nsb = p.n_rows[kSolid] * nch;
-    const bool water = b >= nsb;
-    const int bb = water ? b - nsb : b;
+    const int nch = p.snchunk, nsb = p.n_rows[kSolid] * nch, nss = p.split ? 2 * nsb : nsb;
+    const bool water = b >= nss;
+    int bb = water ? b - nss : b;
+    int species = 0;  // solid blocks: 0 both, 1 electrons, 2 phonons
+    if (!water && p.split) {
+        species = bb >= nsb ? 2 : 1;
+        bb -= (species - 1) * nsb;
+    }
     int row = bb / nch;
-    int x = (bb - row * nch) * blockDim.x + threadIdx.x;
-    const int x_lane = x;
+    const int x = (bb - row * nch) * blockDim.x + threadIdx.x;
     bool live = x < p.nx;
-    if constexpr (KLB_BOUNDS) {
-        if (live && !row_indices_ok<Q>(p, water, row, 0, x)) {
-            live = false;
-            row = 0;
-        }
-    }
-    if constexpr (!ACC) {
-        if (!live) return;  // no warp-wide operation follows
-    } else {
-        if (!live) x = 0;   // computes nothing, but joins the warp reduction
-    }
+    if constexpr (KLB_BOUNDS) live = live && row_indices_ok<Q>(p, water, row, 0, x);
+    if (!live) return;
     const int pm = x == 0 ? p.nx - 1 : x - 1;
     const int pp = x == p.nx - 1 ? 0 : x + 1;
     const int nxp = p.nxp;
-    const float inv = p.inv_scale, sc = p.scale;
+    const S inv = 1, sc = 1;
 
     const RowInfo &R = p.rows[water ? kFluid : kSolid][row];
     const int4 *t4 = reinterpret_cast<const int4 *>(&R);
@@ -957,75 +1003,40 @@ __device__ __forceinline__ void step_body(const StepArgs<T> &p, int b)
     if (water) {
         T g[Q], j[3];
         Cell<T> c;
-        if (!ACC || live) {
-            pull_row<Q, T, S>(static_cast<const S *>(p.in[0]), src, xm, xp, xbounce, x, pm, pp,
-                              ref_row<T, S>(p.dec_in[0], row), inv, g);
-            water_math<Q, T>(p, p.U1[kFluid], p.U2[kFluid], p.U1[kSolid], p.U2[kSolid], R, x, g, c, j);
-            if (q5.y >= 0) {
-                const int ns = p.n_slots[kFluid];
-                for (int a = 0; a < 3; ++a) p.U0[kFluid][(a * ns + q5.y) * nxp + x] = c.u[a];
-            }
-            collide<Q, T>(g, c, j, p.rho0, p.om[0]);
-            if constexpr (NOISE)
-                thermal_noise<Q, T>(p, (uint32_t)x + (uint32_t)p.nx * (uint32_t)q7.y,
-                                    [&](int i, T v) { g[i] += v; });
-            store_cell<Q, T, S>(g, static_cast<S *>(p.out[0]), p.n_rows[kFluid] * nxp,
-                                row * nxp + x, ref_row<T, S>(p.enc_out[0], row), sc);
+        pull_row<Q, T, S>(static_cast<const S *>(p.in[0]), src, xm, xp, xbounce, x, pm, pp, nullptr, inv, g);
+        water_math<Q, T>(p, p.U1[kFluid], p.U2[kFluid], p.U1[kSolid], p.U2[kSolid], R, x, g, c, j);
+        if (q5.y >= 0) {
+            const int ns = p.n_slots[kFluid];
+            for (int a = 0; a < 3; ++a) p.U0[kFluid][(a * ns + q5.y) * nxp + x] = c.u[a];
         }
-        if constexpr (ACC) {
-            float acc[2 * Q];
-#pragma unroll
-            for (int i = 0; i < Q; ++i) {
-                acc[i] = live ? float(g[i]) : 0.f;
-                acc[Q + i] = 0.f;
-            }
-            const int seg = warp_segment(p, true, row, x_lane);
-            if (seg >= 0) warp_xsum<2 * Q>(acc, p.acc + (size_t)seg * 2 * Q);
-        }
+        collide<Q, T>(g, c, j, p.rho0, p.om[0]);
+        if constexpr (NOISE)
+            thermal_noise<Q, T>(p, (uint32_t)x + (uint32_t)p.nx * (uint32_t)q7.y, [&](int i, T v) { g[i] += v; });
+        store_cell<Q, T, S>(g, static_cast<S *>(p.out[0]), p.n_rows[kFluid] * nxp, row * nxp + x, nullptr, sc);
         return;
     }
 
+    // With `split` (FP64 lattices too small to fill the chip) a block keeps
+    // one species of its row: it streams both, for the coupled velocities.
     T ge[Q], gp[Q], je[3], jp[3];
     Cell<T> ce, cp;
-    float acc[ACC ? 2 * Q : 1];
-    if (!ACC || live) {
-        pull_row<Q, T, S>(static_cast<const S *>(p.in[1]), src, xm, xp, xbounce, x, pm, pp,
-                          ref_row<T, S>(p.dec_in[1], row), inv, ge);
-        pull_row<Q, T, S>(static_cast<const S *>(p.in[2]), src, xm, xp, xbounce, x, pm, pp,
-                          ref_row<T, S>(p.dec_in[2], row), inv, gp);
-        solid_math<Q, T>(p, p.U1[kFluid], p.U2[kFluid], p.U1[kSolid], p.U2[kSolid], R, x, ge, gp,
-                         ce, cp, je, jp);
-        if (q5.y >= 0) {
-            const int ns = p.n_slots[kSolid];
-            for (int a = 0; a < 3; ++a) {
-                p.U0[kSolid][(a * ns + q5.y) * nxp + x] = ce.u[a];
-                p.U0[kSolid][((a + 3) * ns + q5.y) * nxp + x] = cp.u[a];
-            }
-        }
-        const int stride = p.n_rows[kSolid] * nxp, base = row * nxp + x;
+    pull_row<Q, T, S>(static_cast<const S *>(p.in[1]), src, xm, xp, xbounce, x, pm, pp, nullptr, inv, ge);
+    pull_row<Q, T, S>(static_cast<const S *>(p.in[2]), src, xm, xp, xbounce, x, pm, pp, nullptr, inv, gp);
+    solid_math<Q, T>(p, p.U1[kFluid], p.U2[kFluid], p.U1[kSolid], p.U2[kSolid], R, x, ge, gp, ce, cp, je, jp);
+    const int stride = p.n_rows[kSolid] * nxp, base = row * nxp + x, ns = p.n_slots[kSolid];
+    if (species != 2) {
+        if (q5.y >= 0)
+            for (int a = 0; a < 3; ++a) p.U0[kSolid][(a * ns + q5.y) * nxp + x] = ce.u[a];
         collide<Q, T>(ge, ce, je, p.rho0, p.om[1]);
-        store_cell<Q, T, S>(ge, static_cast<S *>(p.out[1]), stride, base,
-                            ref_row<T, S>(p.enc_out[1], row), sc);
-        if constexpr (ACC) {
-#pragma unroll
-            for (int i = 0; i < Q; ++i) acc[i] = float(ge[i]);
-        }
-        pull_row<Q, T, S>(static_cast<const S *>(p.in[2]), src, xm, xp, xbounce, x, pm, pp,
-                          ref_row<T, S>(p.dec_in[2], row), inv, gp);
-        collide<Q, T>(gp, cp, jp, p.rho0, p.om[2], p.q_p);
-        store_cell<Q, T, S>(gp, static_cast<S *>(p.out[2]), stride, base,
-                            ref_row<T, S>(p.enc_out[2], row), sc);
-        if constexpr (ACC) {
-#pragma unroll
-            for (int i = 0; i < Q; ++i) acc[Q + i] = float(gp[i]);
-        }
-    } else if constexpr (ACC) {
-#pragma unroll
-        for (int k = 0; k < 2 * Q; ++k) acc[k] = 0.f;
+        store_cell<Q, T, S>(ge, static_cast<S *>(p.out[1]), stride, base, nullptr, sc);
     }
-    if constexpr (ACC) {
-        const int seg = warp_segment(p, false, row, x_lane);
-        if (seg >= 0) warp_xsum<2 * Q>(acc, p.acc + (size_t)seg * 2 * Q);
+    if (species != 1) {
+        if (q5.y >= 0)
+            for (int a = 0; a < 3; ++a) p.U0[kSolid][((a + 3) * ns + q5.y) * nxp + x] = cp.u[a];
+        if (species == 0)
+            pull_row<Q, T, S>(static_cast<const S *>(p.in[2]), src, xm, xp, xbounce, x, pm, pp, nullptr, inv, gp);
+        collide<Q, T>(gp, cp, jp, p.rho0, p.om[2], p.q_p);
+        store_cell<Q, T, S>(gp, static_cast<S *>(p.out[2]), stride, base, nullptr, sc);
     }
 }
 
@@ -1036,20 +1047,20 @@ __device__ __forceinline__ void step_body(const StepArgs<T> &p, int b)
 namespace klb {
 
 // FP32 arithmetic: two cells per thread (klb_step_pair.cuh); FP64: one.
-template <int Q, typename T, typename S, bool ACC, bool NOISE = false>
+template <int Q, typename T, typename S, bool ACC, bool NOISE, bool EP>
 __device__ __forceinline__ void step_cells_body(const StepArgs<T> &p, int b)
 {
     if constexpr (sizeof(T) == 4)
-        step_body2<Q, S, ACC, NOISE>(p, b);
+        step_body2<Q, S, ACC, NOISE, EP>(p, b);
     else
-        step_body<Q, T, S, ACC, NOISE>(p, b);
+        step_body<Q, T, S, NOISE>(p, b);
 }
 
-template <int Q, typename T, typename S, bool ACC, bool NOISE = false>
-__global__ void __launch_bounds__(kBlockX, (step_min_blocks<T, S>())) k_step(const StepArgs<T> p)
+template <int Q, typename T, typename S, bool ACC, bool NOISE = false, bool EP = false>
+__global__ void __launch_bounds__(kBlockX, (step_min_blocks<T, S, EP>())) k_step(const StepArgs<T> p)
 {
     pdl_launch_dependents();
-    step_cells_body<Q, T, S, ACC, NOISE>(p, blockIdx.x);
+    step_cells_body<Q, T, S, ACC, NOISE, EP>(p, blockIdx.x);
 }
 
 // Launch of a step kernel that may begin while the previous kernel of the
@@ -1076,8 +1087,8 @@ cudaError_t launch_step(void (*kernel)(A), int nblocks, int bx, cudaStream_t s, 
 // independent loads, no block barrier: the latency is before everything
 // else), and the block works from a shared-memory copy of that lattice's
 // arguments.
-template <int Q, typename T, typename S, bool ACC>
-__global__ void __launch_bounds__(kBlockX, (step_min_blocks<T, S>()))
+template <int Q, typename T, typename S, bool ACC, bool EP>
+__global__ void __launch_bounds__(kBlockX, (step_min_blocks<T, S, EP>()))
     k_step_batch(const StepArgs<T> *__restrict__ table, const int *__restrict__ prefix, int n)
 {
     pdl_launch_dependents();
@@ -1090,7 +1101,7 @@ __global__ void __launch_bounds__(kBlockX, (step_min_blocks<T, S>()))
     int4 *dst = reinterpret_cast<int4 *>(&sp);
     for (int k = threadIdx.x; k < (int)(sizeof(StepArgs<T>) / 16); k += blockDim.x) dst[k] = __ldg(src + k);
     __syncthreads();
-    step_cells_body<Q, T, S, ACC>(sp, (int)blockIdx.x - __ldg(prefix + lid));
+    step_cells_body<Q, T, S, ACC, false, EP>(sp, (int)blockIdx.x - __ldg(prefix + lid));
 }
 
 // ---------------------------------------------------------------------------
@@ -1161,6 +1172,16 @@ cudaError_t launch_q(const void *args, int mode, int nblocks, int bx, cudaStream
             return launch_step<StepArgs<T>>(k_step<Q, T, S, true>, nblocks, bx, s, a);
         else
             return cudaErrorInvalidValue;
+    case kModeStepEp:
+        if constexpr (sizeof(T) == 4)
+            return launch_step<StepArgs<T>>(k_step<Q, T, S, false, false, true>, nblocks, bx, s, a);
+        else
+            return cudaErrorInvalidValue;
+    case kModeStepAccEp:
+        if constexpr (Storage<S>::kRef)
+            return launch_step<StepArgs<T>>(k_step<Q, T, S, true, false, true>, nblocks, bx, s, a);
+        else
+            return cudaErrorInvalidValue;
     case kModeStepNoise:
         if constexpr (!Storage<S>::kRef)
             return launch_step<StepArgs<T>>(k_step<Q, T, S, false, true>, nblocks, bx, s, a);
@@ -1194,7 +1215,7 @@ cudaError_t launch_q(const void *args, int mode, int nblocks, int bx, cudaStream
 
 template <int Q, typename T, typename S>
 cudaError_t launch_batch_q(const void *table, const int *prefix, int n, int nblocks, int bx,
-                           bool acc, cudaStream_t s)
+                           bool acc, bool ep, cudaStream_t s)
 {
     const StepArgs<T> *t = static_cast<const StepArgs<T> *>(table);
     cudaLaunchConfig_t cfg = {};
@@ -1206,13 +1227,16 @@ cudaError_t launch_batch_q(const void *table, const int *prefix, int n, int nblo
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (acc) {
-        if constexpr (Storage<S>::kRef)
-            return cudaLaunchKernelEx(&cfg, k_step_batch<Q, T, S, true>, t, prefix, n);
-        else
-            return cudaErrorInvalidValue;
+    if constexpr (Storage<S>::kRef) {
+        if (acc)
+            return ep ? cudaLaunchKernelEx(&cfg, k_step_batch<Q, T, S, true, true>, t, prefix, n)
+                      : cudaLaunchKernelEx(&cfg, k_step_batch<Q, T, S, true, false>, t, prefix, n);
     }
-    return cudaLaunchKernelEx(&cfg, k_step_batch<Q, T, S, false>, t, prefix, n);
+    if (acc) return cudaErrorInvalidValue;
+    if constexpr (sizeof(T) == 4) {
+        if (ep) return cudaLaunchKernelEx(&cfg, k_step_batch<Q, T, S, false, true>, t, prefix, n);
+    }
+    return cudaLaunchKernelEx(&cfg, k_step_batch<Q, T, S, false, false>, t, prefix, n);
 }
 
 template <int Q, typename T>

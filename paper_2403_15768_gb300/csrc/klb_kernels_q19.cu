@@ -1,9 +1,14 @@
 // Instantiations of the KLB kernels for the D3Q19 lattice (templates in
-// klb_kernels.cuh).
+// klb_kernels.cuh) with FP64 and FP32 storage; 16-bit storage in
+// klb_kernels_q19_16.cu, so that the two compile in parallel.
 
 #include "klb_kernels.cuh"
 
 namespace klb {
+
+cudaError_t launch_q19_16(int storage, const void *args, int mode, int nblocks, int bx, cudaStream_t s);
+cudaError_t launch_batch_q19_16(int storage, const void *table, const int *prefix, int n, int nblocks,
+                                int bx, bool acc, bool ep, cudaStream_t s);
 
 cudaError_t launch_q19(int storage, const void *args, int mode, int nblocks, int bx, cudaStream_t s)
 {
@@ -12,34 +17,21 @@ cudaError_t launch_q19(int storage, const void *args, int mode, int nblocks, int
         return launch_q<19, double, double>(args, mode, nblocks, bx, s);
     case KLB_FP32:
         return launch_q<19, float, float>(args, mode, nblocks, bx, s);
-    case KLB_FP16_DEV:
-        return launch_q<19, float, __half>(args, mode, nblocks, bx, s);
-    case KLB_BF16_DEV:
-        return launch_q<19, float, __nv_bfloat16>(args, mode, nblocks, bx, s);
     default:
-        return cudaErrorInvalidValue;
+        return launch_q19_16(storage, args, mode, nblocks, bx, s);
     }
 }
 
-cudaError_t launch_ref_q19(const void *args, float *const enc[3], float *const dec[3], cudaStream_t s)
-{
-    return launch_ref_q<19, float>(args, enc, dec, s);
-}
-
 cudaError_t launch_batch_q19(int storage, const void *table, const int *prefix, int n, int nblocks,
-                          int bx, bool acc, cudaStream_t s)
+                          int bx, bool acc, bool ep, cudaStream_t s)
 {
     switch (storage) {
     case KLB_FP64:
-        return launch_batch_q<19, double, double>(table, prefix, n, nblocks, bx, acc, s);
+        return launch_batch_q<19, double, double>(table, prefix, n, nblocks, bx, acc, ep, s);
     case KLB_FP32:
-        return launch_batch_q<19, float, float>(table, prefix, n, nblocks, bx, acc, s);
-    case KLB_FP16_DEV:
-        return launch_batch_q<19, float, __half>(table, prefix, n, nblocks, bx, acc, s);
-    case KLB_BF16_DEV:
-        return launch_batch_q<19, float, __nv_bfloat16>(table, prefix, n, nblocks, bx, acc, s);
+        return launch_batch_q<19, float, float>(table, prefix, n, nblocks, bx, acc, ep, s);
     default:
-        return cudaErrorInvalidValue;
+        return launch_batch_q19_16(storage, table, prefix, n, nblocks, bx, acc, ep, s);
     }
 }
 

@@ -413,6 +413,151 @@ __device__ __forceinline__ void collide2(float2 g[Q], const Cell2 &c, const floa
     }
 }
 
+// ---------------------------------------------------------------------------
+// Species pairs: one solid cell per thread, its electrons (x) and phonons (y)
+// as the packed pair.  The operations on each element are those of the cell
+// pairs above, so the results are the same bits; relaxation rate, second-order
+// factor and dither differ between the elements.  See step_ep for when.
+
+template <int Q, bool DITHER>
+__device__ __forceinline__ void collide_ep(float2 g[Q], const Cell2 &c, const float2 j[3], float rho0,
+                                           float2 om, float2 q, uint2 sd)
+{
+    const float2 rho = add2(b2(rho0), c.drho);
+    const float2 uu = fma2(c.u[2], c.u[2], fma2(c.u[1], c.u[1], mul2(c.u[0], c.u[0])));
+    const float2 uF = fma2(c.u[2], c.F[2], fma2(c.u[1], c.F[1], mul2(c.u[0], c.F[0])));
+    const float2 e0 = fma2(mul2(mul2(b2(-1.5f), q), rho), uu, c.drho);
+    const float2 r45 = mul2(mul2(b2(4.5f), q), rho);
+    const float2 m3uF = mul2(mul2(b2(-3.f), q), uF);
+    const float2 q9 = mul2(b2(9.f), q);
+    const float2 om1 = sub2(b2(1.f), om), fo = sub2(b2(1.f), mul2(b2(0.5f), om));
+    float2 dm = b2(0.f), dj[3] = {b2(0.f), b2(0.f), b2(0.f)};
+    {
+        const float w = float(wt<Q>(0));
+        const float2 g0 = g[0];
+        g[0] = fma2(om1, g[0], fma2(mul2(om, b2(w)), e0, mul2(mul2(fo, b2(w)), m3uF)));
+        if constexpr (DITHER) dm = sub2(g0, g[0]);
+    }
+#pragma unroll
+    for (int i = 1; i < Q; ++i) {
+        if (opp<Q>(i) < i) continue;
+        const int ib = opp<Q>(i);
+        const float w = float(wt<Q>(i));
+        const float2 cu = cdot2<Q>(i, c.u);
+        const float2 cF = cdot2<Q>(i, c.F);
+        const float2 se = fma2(r45, mul2(cu, cu), e0);
+        const float2 sf = fma2(q9, mul2(cu, cF), m3uF);
+        const float2 ow = mul2(om, b2(w)), fw = mul2(fo, b2(w));
+        const float2 S = fma2(ow, se, mul2(fw, sf));
+        const float2 A = fma2(mul2(mul2(mul2(b2(3.f), om), b2(w)), rho), cu, mul2(mul2(mul2(b2(3.f), fo), b2(w)), cF));
+        const float2 gi = g[i], gb = g[ib];
+        g[i] = fma2(om1, gi, add2(S, A));
+        g[ib] = fma2(om1, gb, sub2(S, A));
+        if constexpr (DITHER) {
+            const float2 di = sub2(gi, g[i]), db = sub2(gb, g[ib]);
+            dm = add2(dm, add2(di, db));
+            const float2 dd = sub2(di, db);
+            const int cc[3] = {cx<Q>(i), cy<Q>(i), cz<Q>(i)};
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                if (cc[k] > 0) dj[k] = add2(dj[k], dd);
+                if (cc[k] < 0) dj[k] = sub2(dj[k], dd);
+            }
+        }
+    }
+    if constexpr (DITHER) {
+        auto dither = [&](float2 a, float2 b, uint32_t m) {
+            return add2(a, add2(b, make_float2(dither_unit(sd.x * m) * ulp_of(a.x), dither_unit(sd.y * m) * ulp_of(a.y))));
+        };
+        g[0] = dither(g[0], dm, 1u);
+#pragma unroll
+        for (int k = 0; k < (Q == 19 ? 3 : 2); ++k) {
+            const float2 h = mul2(b2(0.5f), add2(dj[k], c.F[k]));
+            const int ip = dir_index<Q>(k == 0, k == 1, k == 2);
+            const int im = dir_index<Q>(-(k == 0), -(k == 1), -(k == 2));
+            const uint32_t mp = 0x9E3779B9u * (uint32_t)(2 * k + 1) | 1u, mm = 0x9E3779B9u * (uint32_t)(2 * k + 2) | 1u;
+            g[ip] = dither(g[ip], h, mp);
+            g[im] = dither(g[im], make_float2(-h.x, -h.y), mm);
+        }
+        return;
+    }
+    float2 m, pm[3];
+    moments2<Q>(g, m, pm);
+    g[0] = add2(g[0], sub2(c.drho, m));
+#pragma unroll
+    for (int k = 0; k < (Q == 19 ? 3 : 2); ++k) {
+        const float2 h = mul2(b2(0.5f), add2(sub2(j[k], pm[k]), c.F[k]));
+        const int ip = dir_index<Q>(k == 0, k == 1, k == 2);
+        const int im = dir_index<Q>(-(k == 0), -(k == 1), -(k == 2));
+        g[ip] = add2(g[ip], h);
+        g[im] = sub2(g[im], h);
+    }
+}
+
+// Pull of one solid cell (columns as in pull_cols).
+template <int Q, typename S, bool XB>
+__device__ __forceinline__ void pull_ep(const S *__restrict__ ie, const S *__restrict__ ip, const int src[Q],
+                                        uint32_t moves, int x, int xm, int xp, const float *de, const float *dp,
+                                        float inv, float2 g[Q])
+{
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        int a = cx<Q>(i) > 0 ? xm : (cx<Q>(i) < 0 ? xp : x);
+        if constexpr (XB) {
+            if (cx<Q>(i) != 0) a = ((moves >> i) & 1u) ? a : x;
+        }
+        g[i] = make_float2(Pair<S>::load1(src_row(ie, src[i]) + a), Pair<S>::load1(src_row(ip, src[i]) + a));
+    }
+    if constexpr (Storage<S>::kRef) {
+#pragma unroll
+        for (int i = 0; i < Q; ++i) g[i] = fma2(g[i], b2(inv), make_float2(__ldg(de + i), __ldg(dp + i)));
+    }
+}
+
+__device__ __forceinline__ float lagged1(const float *U1, const float *U2, int idx)
+{
+    return __fmul_rn(0.5f, __fadd_rn(U1[idx], U2[idx]));
+}
+
+template <int Q>
+__device__ __forceinline__ void solid_math_ep(const StepArgs<float> &p, const RowInfo &R, int x, const float2 g[Q],
+                                              Cell2 &c, float2 j[3])
+{
+    moments2<Q>(g, c.drho, j);
+    float2 F[3] = {b2(0.f), b2(0.f), b2(0.f)};
+    const int slot = R.slot;
+    if (slot >= 0) {
+        const float *Uw1 = p.U1[kFluid], *Uw2 = p.U2[kFluid], *Us1 = p.U1[kSolid], *Us2 = p.U2[kSolid];
+        const int ns_w = p.n_slots[kFluid], ns_s = p.n_slots[kSolid], nxp = p.nxp;
+        const int nface = R.nface;
+        float2 us[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+            us[a] = make_float2(lagged1(Us1, Us2, (a * ns_s + slot) * nxp + x), lagged1(Us1, Us2, ((a + 3) * ns_s + slot) * nxp + x));
+#pragma unroll 1
+        for (int k = 0; k < nface; ++k) {
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const float uw = lagged1(Uw1, Uw2, (a * ns_w + R.partner[k]) * nxp + x);
+                F[a] = fma2(make_float2(p.g_we, p.g_wp), sub2(b2(uw), us[a]), F[a]);
+            }
+        }
+    }
+    const float k = 0.5f * p.g_ep, se = 0.5f * p.g_ec, sp = 0.5f * p.g_pc;
+    const float2 AB = add2(add2(b2(p.rho0), c.drho), make_float2(k + se, k + sp));
+    const float2 BA = make_float2(AB.y, AB.x);
+    const float Dinv = 1.f / __fsub_rn(__fmul_rn(AB.x, AB.y), k * k);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const float2 J = fma2(b2(0.5f), F[a], j[a]);
+        const float2 u = mul2(fma2(BA, J, mul2(b2(k), make_float2(J.y, J.x))), b2(Dinv));
+        c.u[a] = u;
+        const float d = __fsub_rn(u.x, u.y);
+        const float2 s = mul2(make_float2(p.g_ec, p.g_pc), u);
+        c.F[a] = sub2(make_float2(__fsub_rn(F[a].x, __fmul_rn(p.g_ep, d)), __fmaf_rn(p.g_ep, d, F[a].y)), s);
+    }
+}
+
 // Store g* of both cells, encoded against the row's references for 16-bit
 // storage: (g - ref) * scale = fma(g, scale, -ref * scale) exactly, scale
 // being a power of two.  The second cell of an odd row's last pair goes to
@@ -495,7 +640,7 @@ __device__ __forceinline__ void prefetch_rows(const StepArgs<float> &p, bool wat
     }
 }
 
-template <int Q, typename S, bool ACC, bool NOISE = false>
+template <int Q, typename S, bool ACC, bool NOISE, bool EP>
 __device__ __forceinline__ void step_body2(const StepArgs<float> &p, int b)
 {
     // An item is 64 cells of a row, one per warp; solid items (two species
@@ -507,20 +652,21 @@ __device__ __forceinline__ void step_body2(const StepArgs<float> &p, int b)
     // per row chunk, one-warp blocks for narrow rows, and a division for the
     // row: 301x77x93 slab 66.3 us (now 64.4), 193x97x97 BF16 48.0 (47.0),
     // 12-channel sweep FP32 480.8 (475.3), FP16 457.1 (439.1).
-    const int nseg = p.nseg64, nsi = p.n_rows[kSolid] * nseg;
+    const int nsi = p.n_rows[kSolid] * p.sseg;
     const int it = (int)__reduce_max_sync(0xffffffffu, (unsigned)(b * ((int)blockDim.x >> 5) + ((int)threadIdx.x >> 5)));
     const bool water = it >= nsi;
     const int ii = water ? it - nsi : it;
-    int row = (int)(((unsigned long long)(unsigned)ii * p.seg_mul) >> p.seg_shift);
+    int row = (int)(((unsigned long long)(unsigned)ii * (water ? p.seg_mul : p.sseg_mul)) >> (water ? p.seg_shift : p.sseg_shift));
     if (water && row >= p.n_rows[kFluid]) return;
-    const int sg = ii - row * nseg;  // segment
-    if constexpr (!NOISE) {
+    const int sg = ii - row * (water ? p.nseg64 : p.sseg);  // segment
+    if constexpr (!NOISE && !EP) {
         if (p.ahead) prefetch_rows<Q, S>(p, water, row, sg);
     }
-    const int x_first = 64 * sg + 2 * ((int)threadIdx.x & 31);
+    const bool one = EP && !water;  // one cell per thread
+    const int x_first = one ? 32 * sg + ((int)threadIdx.x & 31) : 64 * sg + 2 * ((int)threadIdx.x & 31);
     bool live = x_first < p.nx;
     if constexpr (KLB_BOUNDS) {
-        if (live && !row_indices_ok<Q>(p, water, row, 0, x_first + 1)) {
+        if (live && !row_indices_ok<Q>(p, water, row, 0, one ? x_first : x_first + 1)) {
             live = false;
             row = 0;
         }
@@ -554,7 +700,7 @@ __device__ __forceinline__ void step_body2(const StepArgs<float> &p, int b)
     const uint32_t xp = (uint32_t)q5.x;
     const bool xbounce = (q7.x & kXBounce) != 0;
 
-    const int seg = ACC ? thread_segment<2>(p, water, row, x_first) : -1;
+    const int seg = !ACC ? -1 : one ? thread_segment<1>(p, water, row, x_first) : thread_segment<2>(p, water, row, x_first);
     pdl_wait();  // populations, lagged velocities, references and the period count below
     constexpr bool DITHER = !Storage<S>::kRef;
     const uint32_t n_step = p.step_lo + (p.step_reps ? *p.step_reps * (uint32_t)p.step_period : 0u);
@@ -590,6 +736,58 @@ __device__ __forceinline__ void step_body2(const StepArgs<float> &p, int b)
         return;
     }
 
+    if constexpr (EP) {
+        float2 g[Q], j[3];
+        Cell2 c;
+        const S *ie = static_cast<const S *>(p.in[1]), *ip = static_cast<const S *>(p.in[2]);
+        const float *de = ref_row<float, S>(p.dec_in[1], row), *dp = ref_row<float, S>(p.dec_in[2], row);
+        if (!xbounce)
+            pull_ep<Q, S, false>(ie, ip, src, 0u, X.x0, X.pm_a, X.pp_a, de, dp, inv, g);
+        else
+            pull_ep<Q, S, true>(ie, ip, src, xm | xp, X.x0, X.pm_a, X.pp_a, de, dp, inv, g);
+        solid_math_ep<Q>(p, R, X.x0, g, c, j);
+        if (q5.y >= 0 && live) {
+            const int ns = p.n_slots[kSolid];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                p.U0[kSolid][(a * ns + q5.y) * nxp + X.x0] = c.u[a].x;
+                p.U0[kSolid][((a + 3) * ns + q5.y) * nxp + X.x0] = c.u[a].y;
+            }
+        }
+        collide_ep<Q, DITHER>(g, c, j, p.rho0, make_float2(p.om[1], p.om[2]), make_float2(1.f, p.q_p),
+                              make_uint2(dither_seed((uint32_t)q7.y, n_step, 1), dither_seed((uint32_t)q7.y, n_step, 2)));
+        if (live) {
+            const int stride = p.n_rows[kSolid] * nxp, base = row * nxp + X.x0;
+            S *oe = static_cast<S *>(p.out[1]), *op = static_cast<S *>(p.out[2]);
+            const float *ee = ref_row<float, S>(p.enc_out[1], row), *ep = ref_row<float, S>(p.enc_out[2], row);
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                float2 v = g[i];
+                if constexpr (Storage<S>::kRef) v = fma2(v, b2(sc), make_float2(-__ldg(ee + i) * sc, -__ldg(ep + i) * sc));
+                const long long o = (long long)i * stride + base;
+                Storage<S>::store(oe + o, v.x);
+                Storage<S>::store(op + o, v.y);
+            }
+        }
+        if constexpr (ACC) {
+            float acc[2 * Q];
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                acc[i] = live ? g[i].x : 0.f;
+                acc[Q + i] = live ? g[i].y : 0.f;
+            }
+            const int lane = threadIdx.x & 31;
+#pragma unroll
+            for (int k = 0; k < 2 * Q; ++k) {
+                float v = acc[k];
+                v += __shfl_xor_sync(0xffffffffu, v, 1);
+#pragma unroll
+                for (int o = 16; o > 1; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                if (lane == 0 && seg >= 0) p.acc[(size_t)seg * 2 * Q + k] = v;
+            }
+        }
+        return;
+    }
     float2 ge[Q], gp[Q], je[3], jp[3];
     Cell2 ce, cp;
     pull_row2<Q, S>(static_cast<const S *>(p.in[1]), src, xm, xp, xbounce, X,
