@@ -91,7 +91,7 @@ size_t state_bytes(const klb_lattice *L)
 // one observed); the step kernel runs blocks of sbx threads and touches
 // all_bytes of state buffers per launch.
 template <typename T>
-void fill_args_at(const klb_lattice *L, const HostState &st, int sbx, size_t all_bytes, StepArgs<T> &a)
+void fill_args_at(const klb_lattice *L, const HostState &st, int sbx, bool ep, size_t all_bytes, StepArgs<T> &a)
 {
     const Geometry &g = L->geo;
     const MemoryPlan &p = L->plan;
@@ -128,13 +128,18 @@ void fill_args_at(const klb_lattice *L, const HostState &st, int sbx, size_t all
     a.nchunk = p.nchunk;
     a.nbw = (int)g.rows[kFluid].size() * a.nchunk;
     a.snchunk = (g.nx + sbx - 1) / sbx;
+    a.split = L->desc.storage == KLB_FP64 && fp64_split(g.nx, a.n_rows[kFluid], a.n_rows[kSolid]);
+    // divisions by multiplication: the kernel's first instructions wait for them
+    auto divider = [](int d, uint32_t &mul, uint32_t &shift) {
+        uint32_t sh = 0;
+        while ((1u << sh) < (uint32_t)d) ++sh;
+        shift = 31 + sh;
+        mul = (uint32_t)((1ull << (31 + sh)) / (uint32_t)d + 1);
+    };
     a.nseg64 = (g.nx + 63) / 64;
-    {
-        uint32_t sh = 0;  // division by multiplication: the kernel's first instructions wait for it
-        while ((1u << sh) < (uint32_t)a.nseg64) ++sh;
-        a.seg_shift = 31 + sh;
-        a.seg_mul = (uint32_t)((1ull << (31 + sh)) / (uint32_t)a.nseg64 + 1);
-    }
+    a.sseg = ep ? (g.nx + 31) / 32 : a.nseg64;
+    divider(a.nseg64, a.seg_mul, a.seg_shift);
+    divider(a.sseg, a.sseg_mul, a.sseg_shift);
     a.nch32 = (g.nx + 31) / 32;
     a.nseg_w = (int)g.rows[kFluid].size() * a.nch32;
     const klb_desc &d = L->desc;
@@ -165,7 +170,7 @@ void fill_args_at(const klb_lattice *L, const HostState &st, int sbx, size_t all
 template <typename T>
 void fill_args(const klb_lattice *L, StepArgs<T> &a)
 {
-    fill_args_at(L, L->st, L->plan.sbx, state_bytes(L), a);
+    fill_args_at(L, L->st, L->plan.sbx, L->plan.ep, state_bytes(L), a);
 }
 
 // The host side of one step: encode generation of the output, whether the
@@ -544,7 +549,7 @@ klb_status klb_step(klb_lattice *L, int64_t nsteps)
         cudaError_t e = with_args(L, [&](void *a) {
             set_enc(L, a, sp.outgen);
             const int mode = sp.acc ? kModeStepAcc : (L->kT > 0.0 ? kModeStepNoise : kModeStep);
-            return launch(L->geo.Q, L->desc.storage, a, mode, L->plan.snblocks, L->plan.sbx, L->stream);
+            return launch(L->geo.Q, L->desc.storage, a, L->plan.ep ? mode | kModeEp : mode, L->plan.snblocks, L->plan.sbx, L->stream);
         });
         if (e != cudaSuccess) return cuda_fail(L, e, "step kernel launch");
         advance(L->st, sp);
@@ -878,6 +883,7 @@ struct klb_batch {
     int period = 6;
     int width = kBlockX;
     int nblocks = 0;
+    bool ep = false;
     size_t args_size = 0, table_off = 0, prefix_off = 0, reps_off = 0;
     std::vector<StepPlan> plans;  // per (phase, member)
     std::vector<char> acc;        // per phase: some member accumulates x-sums
@@ -949,13 +955,13 @@ klb_status build_tables(klb_batch *B, int width)
             const uint32_t *reps = (const uint32_t *)(B->base + B->reps_off);
             if (B->storage == KLB_FP64) {
                 StepArgs<double> a;
-                fill_args_at(L, st, width, all_bytes, a);
+                fill_args_at(L, st, width, B->ep, all_bytes, a);
                 a.step_reps = reps;
                 a.step_period = P;
                 std::memcpy(slot, &a, sizeof a);
             } else {
                 StepArgs<float> a;
-                fill_args_at(L, st, width, all_bytes, a);
+                fill_args_at(L, st, width, B->ep, all_bytes, a);
                 a.step_reps = reps;
                 a.step_period = P;
                 if (reduced(L))
@@ -966,7 +972,7 @@ klb_status build_tables(klb_batch *B, int width)
         }
         const int sto = L->desc.storage;
         prefix[m + 1] = prefix[m] + step_blocks(L->geo.nx, (int)L->geo.rows[kFluid].size(),
-                                                (int)L->geo.rows[kSolid].size(), width, sto);
+                                                (int)L->geo.rows[kSolid].size(), width, sto, B->ep);
     }
     KLB_BCUDA(B, cudaStreamSynchronize(B->stream));
     KLB_BCUDA(B, cudaMemcpy(B->base + B->table_off, host.data(), host.size(), cudaMemcpyHostToDevice));
@@ -1003,7 +1009,7 @@ cudaError_t launch_phase(klb_batch *B, int k)
     }
     const char *table = B->base + B->table_off + (size_t)k * n * B->args_size;
     cudaError_t e = launch_batch(B->Q, B->storage, table, (const int *)(B->base + B->prefix_off), (int)n,
-                                 B->nblocks, B->width, B->acc[k] != 0, B->stream);
+                                 B->nblocks, B->width, B->acc[k] != 0, B->ep, B->stream);
     if (e == cudaSuccess && k == B->period - 1) e = launch_count_period((uint32_t *)(B->base + B->reps_off), B->stream);
     return e;
 }
@@ -1154,10 +1160,13 @@ klb_status klb_batch_create(klb_lattice *const *members, int n, void *dev_buf, s
     if (B->storage == KLB_FP64) {
         for (klb_lattice *L : B->mem) w = std::min(w, L->plan.sbx);
     } else {
-        long long items = 0;
-        for (klb_lattice *L : B->mem)
-            items += (long long)(L->geo.rows[kFluid].size() + L->geo.rows[kSolid].size()) * ((L->geo.nx + 63) / 64);
-        w = step_width(items);
+        long long items[2] = {0, 0};
+        for (klb_lattice *L : B->mem) {
+            const Geometry &g = L->geo;
+            for (int e = 0; e < 2; ++e) items[e] += step_items(g.nx, g.rows[kFluid].size(), g.rows[kSolid].size(), e != 0);
+        }
+        B->ep = step_ep(items[1]);
+        w = step_width(items[B->ep]);
     }
     klb_status st = build_tables(B, w);
     if (st != KLB_OK) {

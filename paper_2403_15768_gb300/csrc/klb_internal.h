@@ -230,8 +230,7 @@ enum Mode {
     kModeInit = 4,
     kModeInitAcc = 5,  // x-sums of the initial equilibria, nothing stored
     kModeStepNoise = 6, // step with thermal fluctuations of the water
-    kModeStepEp = 7,    // kModeStep and kModeStepAcc with solid items of one cell per thread (step_ep)
-    kModeStepAccEp = 8
+    kModeEp = 8         // added to a step mode: solid items of one cell per thread (step_ep)
 };
 
 // Launchers (return the launch error, if any).

@@ -1172,14 +1172,19 @@ cudaError_t launch_q(const void *args, int mode, int nblocks, int bx, cudaStream
             return launch_step<StepArgs<T>>(k_step<Q, T, S, true>, nblocks, bx, s, a);
         else
             return cudaErrorInvalidValue;
-    case kModeStepEp:
+    case kModeStep | kModeEp:
         if constexpr (sizeof(T) == 4)
             return launch_step<StepArgs<T>>(k_step<Q, T, S, false, false, true>, nblocks, bx, s, a);
         else
             return cudaErrorInvalidValue;
-    case kModeStepAccEp:
+    case kModeStepAcc | kModeEp:
         if constexpr (Storage<S>::kRef)
             return launch_step<StepArgs<T>>(k_step<Q, T, S, true, false, true>, nblocks, bx, s, a);
+        else
+            return cudaErrorInvalidValue;
+    case kModeStepNoise | kModeEp:
+        if constexpr (sizeof(T) == 4 && !Storage<S>::kRef)
+            return launch_step<StepArgs<T>>(k_step<Q, T, S, false, true, true>, nblocks, bx, s, a);
         else
             return cudaErrorInvalidValue;
     case kModeStepNoise:
