@@ -7,8 +7,11 @@
 #include <cstdio>
 #include <cstring>
 #include <limits>
+#include <memory>
 #include <new>
 #include <string>
+#include <system_error>
+#include <thread>
 #include <vector>
 
 #include <cuda_bf16.h>
@@ -72,7 +75,6 @@ klb_status cuda_fail(klb_lattice *L, cudaError_t e, const char *what)
         if (e_ != cudaSuccess) return cuda_fail((L), e_, #call);  \
     } while (0)
 
-size_t pop_size(const klb_lattice *L) { return storage_bytes(L->desc.storage); }
 size_t arith_size(const klb_lattice *L) { return L->desc.storage == KLB_FP64 ? 8 : 4; }
 bool reduced(const klb_lattice *L) { return reduced_storage(L->desc.storage); }
 
@@ -278,26 +280,121 @@ size_t field_offset(const klb_lattice *L, int s)
     return s == 0 ? 0 : 4 * nrw * nxp + (s == 2 ? 4 * nrs * nxp : 0);
 }
 
-template <typename T>
-void host_to_field(const klb_lattice *L, const double *drho, const double *u, std::vector<T> &f)
+// Runs fn(begin, end) over [0, n) on up to 8 host threads, in pieces that
+// touch at least 4 MB of host memory (`bytes` in all); fn must not throw.
+// The host arrays of the box calls are tens of megabytes to gigabytes, and
+// one core reaches a tenth of the memory's bandwidth (128x64x64 checkpoint,
+// 314 MB: 18.2 ms on one core, 8.4 on four, 7.6 on eight, 8.1 on sixteen).
+template <typename F>
+void host_parallel(size_t n, size_t bytes, F fn)
 {
-    const Geometry &g = L->geo;
-    const size_t ncell = (size_t)g.nx * g.ny * g.nz, nxp = g.nxp;
-    f.assign(L->plan.field_bytes / sizeof(T), T(0));
-    for (int s = 0; s < 3; ++s) {
-        const int c = cls_of(s);
-        const size_t nr = g.rows[c].size(), fo = field_offset(L, s);
-        for (size_t r = 0; r < nr; ++r) {
-            const size_t cs = g.rows[c][r];
-            for (int x = 0; x < g.nx; ++x) {
-                const size_t cell = x + (size_t)g.nx * cs;
-                f[fo + r * nxp + x] = drho ? (T)drho[s * ncell + cell] : T(0);
-                for (int a = 0; a < 3; ++a)
-                    f[fo + ((a + 1) * nr + r) * nxp + x] =
-                        u ? (T)u[(s * 3 + a) * ncell + cell] : T(0);
+    constexpr size_t kThreads = 8;
+    size_t k = std::min({n, kThreads, bytes >> 22});
+    if (k > 1) {
+        static const size_t cores = std::max(1u, std::thread::hardware_concurrency());
+        k = std::min(k, cores);
+    }
+    std::thread pool[kThreads];
+    size_t done = 0, started = 0;
+    if (k > 1) {
+        try {
+            for (; started < k - 1; ++started) {
+                const size_t end = n * (started + 1) / k;
+                pool[started] = std::thread(fn, done, end);
+                done = end;
             }
+        } catch (const std::system_error &) {  // no more threads: the rest runs here
         }
     }
+    fn(done, n);
+    for (size_t t = 0; t < started; ++t) pool[t].join();
+}
+
+// Uninitialised host memory for downloads and uploads.
+struct HostBuf {
+    std::unique_ptr<char[]> p;
+    size_t bytes = 0;
+    bool alloc(size_t n)
+    {
+        p.reset(new (std::nothrow) char[n ? n : 1]);
+        bytes = n;
+        return p != nullptr;
+    }
+    template <typename T> T *as() const { return reinterpret_cast<T *>(p.get()); }
+};
+
+// Waits for the stream before the host buffers declared ahead of it are
+// freed, if a call returns before its own synchronisation.
+struct StreamGuard {
+    cudaStream_t s;
+    bool done = false;
+    ~StreamGuard()
+    {
+        if (!done) cudaStreamSynchronize(s);
+    }
+};
+
+klb_status no_host_memory(klb_lattice *L) { return fail(L, KLB_ENOMEM, "host allocation failed"); }
+
+// Rows of host box fields (either may be null) in the layout of the field
+// scratch.
+template <typename T>
+void host_to_field(const klb_lattice *L, const double *drho, const double *u, T *f)
+{
+    const Geometry &g = L->geo;
+    const size_t ncell = (size_t)g.nx * g.ny * g.nz, nxp = g.nxp, nx = g.nx;
+    for (int s = 0; s < 3; ++s) {
+        const int c = cls_of(s);
+        const size_t nr = g.rows[c].size();
+        T *fs = f + field_offset(L, s);
+        host_parallel(nr, nr * nx * 4 * sizeof(double), [&, s, c, nr, fs](size_t r0, size_t r1) {
+            for (int a = 0; a < 4; ++a) {
+                const double *in = a == 0 ? (drho ? drho + s * ncell : nullptr) : (u ? u + (s * 3 + a - 1) * ncell : nullptr);
+                for (size_t r = r0; r < r1; ++r) {
+                    T *o = fs + (a * nr + r) * nxp;
+                    if (!in) {
+                        std::memset((void *)o, 0, nxp * sizeof(T));
+                        continue;
+                    }
+                    const double *q = in + nx * g.rows[c][r];
+                    for (size_t x = 0; x < nx; ++x) o[x] = (T)q[x];
+                    for (size_t x = nx; x < nxp; ++x) o[x] = T(0);
+                }
+            }
+        });
+    }
+}
+
+// Box arrays from rows: plane k of `planes` holds the values row(k, r) -> x
+// of a row class at its cells and 0 elsewhere.
+template <typename F>
+void rows_to_box(const klb_lattice *L, int cls, size_t planes, double *box, F row)
+{
+    const Geometry &g = L->geo;
+    const size_t ncs = (size_t)g.ny * g.nz, nx = g.nx, n = planes * ncs;
+    host_parallel(n, n * nx * sizeof(double), [&, cls, ncs, nx, box](size_t i0, size_t i1) {
+        const int *row_of = g.row_of_cs[cls].data();
+        size_t k = i0 / ncs, cs = i0 - k * ncs;
+        for (size_t i = i0; i < i1;) {
+            double *o = box + i * nx;
+            if (row_of[cs] >= 0) {
+                row(k, (size_t)row_of[cs], o);
+                ++i;
+                ++cs;
+            } else {  // a run of cells without the class
+                const size_t most = std::min(ncs - cs, i1 - i);
+                size_t m = 1;
+                while (m < most && row_of[cs + m] < 0) ++m;
+                std::memset(o, 0, m * nx * sizeof(double));
+                i += m;
+                cs += m;
+            }
+            if (cs == ncs) {
+                cs = 0;
+                ++k;
+            }
+        }
+    });
 }
 
 klb_status sync(klb_lattice *L)
@@ -306,18 +403,54 @@ klb_status sync(klb_lattice *L)
     return KLB_OK;
 }
 
-template <typename T>
-klb_status init_from_fields(klb_lattice *L, const double *drho, const double *u)
+// A state buffer's three species lie one after the other in it, as do the two
+// classes of a lagged-velocity slot: each goes in one copy.
+size_t pops_bytes(const klb_lattice *L)
 {
-    std::vector<T> f;
-    host_to_field<T>(L, drho, u, f);
-    KLB_CUDA(L, cudaMemcpyAsync(dev(L, L->plan.field), f.data(), L->plan.field_bytes,
-                                cudaMemcpyHostToDevice, L->stream));
+    return L->plan.pop[0][2] - L->plan.pop[0][0] + L->plan.pop_bytes[2];
+}
+
+// Start from rest: every population, reference and lagged velocity is 0.
+klb_status init_from_rest(klb_lattice *L)
+{
+    const MemoryPlan &p = L->plan;
+    for (int b = 0; b < 2; ++b)
+        for (int s = 0; s < 3; ++s) KLB_CUDA(L, cudaMemsetAsync(dev(L, p.pop[b][s]), 0, p.pop_bytes[s], L->stream));
+    for (int t = 0; t < 3; ++t)
+        for (int c = 0; c < 2; ++c)
+            if (p.U_bytes[c]) KLB_CUDA(L, cudaMemsetAsync(dev(L, p.U[t][c]), 0, p.U_bytes[c], L->stream));
+    if (reduced(L))
+        for (int s = 0; s < 3; ++s) {
+            KLB_CUDA(L, cudaMemsetAsync(dev(L, p.ref_enc[0][s]), 0, p.ref_bytes[s], L->stream));
+            KLB_CUDA(L, cudaMemsetAsync(dev(L, p.ref_dec[0][s]), 0, p.ref_bytes[s], L->stream));
+        }
+    return KLB_OK;
+}
+
+void reset_state(klb_lattice *L, int64_t step)
+{
     L->st.cur = 0;
-    L->st.step = 0;
+    L->st.step = step;
     L->st.since_reset = 0;
     L->st.gen_buf[0] = L->st.gen_buf[1] = 0;
     L->st.refresh_pending = false;
+}
+
+template <typename T>
+klb_status init_from_fields(klb_lattice *L, const double *drho, const double *u)
+{
+    if (!drho && !u) {
+        reset_state(L, 0);
+        klb_status st = init_from_rest(L);
+        return st != KLB_OK ? st : sync(L);
+    }
+    HostBuf f;
+    StreamGuard guard{L->stream};
+    if (!f.alloc(L->plan.field_bytes)) return no_host_memory(L);
+    host_to_field<T>(L, drho, u, f.as<T>());
+    KLB_CUDA(L, cudaMemcpyAsync(dev(L, L->plan.field), f.p.get(), L->plan.field_bytes,
+                                cudaMemcpyHostToDevice, L->stream));
+    reset_state(L, 0);
     const int slot0 = slot_of(0);
     auto init_pass = [&](int mode) {
         return with_args(L, [&](void *a) {
@@ -342,6 +475,7 @@ klb_status init_from_fields(klb_lattice *L, const double *drho, const double *u)
             if (t != slot0 && L->plan.U_bytes[c])
                 KLB_CUDA(L, cudaMemcpyAsync(dev(L, L->plan.U[t][c]), dev(L, L->plan.U[slot0][c]),
                                             L->plan.U_bytes[c], cudaMemcpyDeviceToDevice, L->stream));
+    guard.done = true;
     return sync(L);
 }
 
@@ -616,31 +750,33 @@ klb_status klb_get_field(klb_lattice *L, double *drho, double *u)
                  return launch(L->geo.Q, L->desc.storage, a, kModeField, nblocks(L),
                                     L->plan.bx, L->stream);
              }));
-    const size_t ts = arith_size(L), nel = L->plan.field_bytes / ts;
-    std::vector<double> f(nel);
-    std::vector<char> raw(L->plan.field_bytes);
-    KLB_CUDA(L, cudaMemcpyAsync(raw.data(), dev(L, L->plan.field), L->plan.field_bytes,
+    HostBuf raw;
+    StreamGuard guard{L->stream};
+    if (!raw.alloc(L->plan.field_bytes)) return no_host_memory(L);
+    KLB_CUDA(L, cudaMemcpyAsync(raw.p.get(), dev(L, L->plan.field), L->plan.field_bytes,
                                 cudaMemcpyDeviceToHost, L->stream));
     klb_status st = sync(L);
+    guard.done = true;
     if (st != KLB_OK) return st;
-    for (size_t k = 0; k < nel; ++k)
-        f[k] = ts == 8 ? ((const double *)raw.data())[k] : (double)((const float *)raw.data())[k];
     const Geometry &g = L->geo;
-    const size_t ncell = (size_t)g.nx * g.ny * g.nz, nxp = g.nxp;
-    if (drho) std::memset(drho, 0, sizeof(double) * 3 * ncell);
-    if (u) std::memset(u, 0, sizeof(double) * 9 * ncell);
-    for (int s = 0; s < 3; ++s) {
-        const int c = cls_of(s);
-        const size_t nr = g.rows[c].size(), fo = field_offset(L, s);
-        for (size_t r = 0; r < nr; ++r)
-            for (int x = 0; x < g.nx; ++x) {
-                const size_t cell = x + (size_t)g.nx * g.rows[c][r];
-                if (drho) drho[s * ncell + cell] = f[fo + r * nxp + x];
-                if (u)
-                    for (int a = 0; a < 3; ++a)
-                        u[(s * 3 + a) * ncell + cell] = f[fo + ((a + 1) * nr + r) * nxp + x];
-            }
-    }
+    const size_t ncell = (size_t)g.nx * g.ny * g.nz, nxp = g.nxp, nx = g.nx;
+    auto put = [&](auto *f) {
+        for (int s = 0; s < 3; ++s) {
+            const int c = cls_of(s);
+            const size_t nr = g.rows[c].size();
+            const auto *fs = f + field_offset(L, s);
+            auto row = [&, fs, nr](size_t a, size_t r, double *o) {
+                const auto *q = fs + (a * nr + r) * nxp;
+                for (size_t x = 0; x < nx; ++x) o[x] = (double)q[x];
+            };
+            if (drho) rows_to_box(L, c, 1, drho + s * ncell, row);
+            if (u) rows_to_box(L, c, 3, u + s * 3 * ncell, [&](size_t a, size_t r, double *o) { row(a + 1, r, o); });
+        }
+    };
+    if (arith_size(L) == 8)
+        put(raw.as<const double>());
+    else
+        put(raw.as<const float>());
     return KLB_OK;
 }
 
@@ -648,85 +784,100 @@ klb_status klb_get_state(klb_lattice *L, double *gout, double *U1, double *U2)
 {
     if (!L) return fail(L, KLB_EINVAL, "null handle");
     const Geometry &g = L->geo;
-    const size_t ps = pop_size(L), ts = arith_size(L), ncell = (size_t)g.nx * g.ny * g.nz,
-                 nxp = g.nxp;
-    const int Q = g.Q;
+    const size_t ncell = (size_t)g.nx * g.ny * g.nz, nxp = g.nxp, nx = g.nx;
+    const int Q = g.Q, storage = L->desc.storage;
     const bool red = reduced(L);
-    const double inv = L->desc.storage == KLB_FP16_DEV ? 1.0 / kFp16Scale : 1.0;
-    // Population value k of a downloaded buffer (reduced storage: the stored
-    // difference, still to be scaled and shifted by its row reference).
-    auto pop = [&](const std::vector<char> &raw, size_t k) -> double {
-        switch (L->desc.storage) {
-        case KLB_FP64:
-            return ((const double *)raw.data())[k];
-        case KLB_FP32:
-            return ((const float *)raw.data())[k];
-        case KLB_FP16_DEV:
-            return (double)__half2float(((const __half *)raw.data())[k]);
-        default:
-            return (double)__bfloat162float(((const __nv_bfloat16 *)raw.data())[k]);
-        }
-    };
-    auto rd = [&](const std::vector<char> &raw, size_t k) {
-        return ts == 8 ? ((const double *)raw.data())[k] : (double)((const float *)raw.data())[k];
-    };
+    const double inv = storage == KLB_FP16_DEV ? 1.0 / kFp16Scale : 1.0;
     if (gout) {
-        std::memset(gout, 0, sizeof(double) * 3 * Q * ncell);
+        HostBuf pops, refs[3];
+        StreamGuard guard{L->stream};
+        const size_t *at = L->plan.pop[L->st.cur];
+        if (!pops.alloc(pops_bytes(L))) return no_host_memory(L);
+        KLB_CUDA(L, cudaMemcpyAsync(pops.p.get(), dev(L, at[0]), pops.bytes, cudaMemcpyDeviceToHost, L->stream));
         for (int s = 0; s < 3; ++s) {
-            std::vector<char> raw(L->plan.pop_bytes[s]);
-            KLB_CUDA(L, cudaMemcpyAsync(raw.data(), dev(L, L->plan.pop[L->st.cur][s]), raw.size(),
-                                        cudaMemcpyDeviceToHost, L->stream));
-            std::vector<float> ref;
-            if (red) {
-                ref.resize(L->plan.ref_bytes[s] / sizeof(float));
-                KLB_CUDA(L, cudaMemcpyAsync(ref.data(), dev(L, L->plan.ref_enc[L->st.gen_buf[L->st.cur]][s]),
-                                            L->plan.ref_bytes[s], cudaMemcpyDeviceToHost, L->stream));
-            }
-            klb_status st = sync(L);
-            if (st != KLB_OK) return st;
+            if (!refs[s].alloc(L->plan.ref_bytes[s])) return no_host_memory(L);
+            if (red)
+                KLB_CUDA(L, cudaMemcpyAsync(refs[s].p.get(), dev(L, L->plan.ref_enc[L->st.gen_buf[L->st.cur]][s]),
+                                            refs[s].bytes, cudaMemcpyDeviceToHost, L->stream));
+        }
+        klb_status st = sync(L);
+        guard.done = true;
+        if (st != KLB_OK) return st;
+        for (int s = 0; s < 3; ++s) {
             const int c = cls_of(s);
             const size_t nr = g.rows[c].size();
-            for (int i = 0; i < Q; ++i)
-                for (size_t r = 0; r < nr; ++r) {
-                    const double shift = red ? (double)ref[r * kRefStride + i] : 0.0;
-                    for (int x = 0; x < g.nx; ++x) {
-                        double v = pop(raw, (i * nr + r) * nxp + x);
-                        if (red) v = (double)(float)(v * inv + shift);
-                        gout[((size_t)s * Q + i) * ncell + x + (size_t)g.nx * g.rows[c][r]] = v;
+            // Population values of a row (reduced storage: the stored
+            // difference, still to be scaled and shifted by its row reference).
+            auto put = [&](auto *pop) {
+                rows_to_box(L, c, Q, gout + (size_t)s * Q * ncell, [&, pop, nr, s](size_t i, size_t r, double *o) {
+                    const auto *q = pop + (i * nr + r) * nxp;
+                    using V = std::decay_t<decltype(*q)>;
+                    if constexpr (std::is_same_v<V, __half> || std::is_same_v<V, __nv_bfloat16>) {
+                        const double shift = refs[s].as<const float>()[r * kRefStride + i];
+                        for (size_t x = 0; x < nx; ++x) {
+                            float v;
+                            if constexpr (std::is_same_v<V, __half>)
+                                v = __half2float(q[x]);
+                            else
+                                v = __bfloat162float(q[x]);
+                            o[x] = (double)(float)((double)v * inv + shift);
+                        }
+                    } else {
+                        for (size_t x = 0; x < nx; ++x) o[x] = (double)q[x];
                     }
-                }
+                });
+            };
+            const char *pop = pops.p.get() + (at[s] - at[0]);
+            switch (storage) {
+            case KLB_FP64:
+                put(reinterpret_cast<const double *>(pop));
+                break;
+            case KLB_FP32:
+                put(reinterpret_cast<const float *>(pop));
+                break;
+            case KLB_FP16_DEV:
+                put(reinterpret_cast<const __half *>(pop));
+                break;
+            default:
+                put(reinterpret_cast<const __nv_bfloat16 *>(pop));
+                break;
+            }
         }
     }
     double *Uo[2] = {U1, U2};
     for (int t = 0; t < 2; ++t) {
         if (!Uo[t]) continue;
-        std::memset(Uo[t], 0, sizeof(double) * 9 * ncell);
         const int slot = slot_of(L->st.step - 1 - t);
-        for (int c = 0; c < 2; ++c) {
-            const size_t ns = g.slot_row[c].size();
-            if (!ns) continue;
-            std::vector<char> raw(L->plan.U_bytes[c]);
-            KLB_CUDA(L, cudaMemcpyAsync(raw.data(), dev(L, L->plan.U[slot][c]), raw.size(),
-                                        cudaMemcpyDeviceToHost, L->stream));
-            klb_status st = sync(L);
-            if (st != KLB_OK) return st;
-            for (size_t q = 0; q < ns; ++q) {
-                const size_t cs = g.rows[c][g.slot_row[c][q]];
-                for (int x = 0; x < g.nx; ++x) {
-                    const size_t cell = x + (size_t)g.nx * cs;
-                    for (int a = 0; a < 3; ++a) {
-                        if (c == kFluid) {
-                            Uo[t][a * ncell + cell] = rd(raw, (a * ns + q) * nxp + x);
-                        } else {
-                            Uo[t][(3 + a) * ncell + cell] = rd(raw, (a * ns + q) * nxp + x);
-                            Uo[t][(6 + a) * ncell + cell] = rd(raw, ((a + 3) * ns + q) * nxp + x);
-                        }
+        HostBuf raw;
+        StreamGuard guard{L->stream};
+        const size_t *at = L->plan.U[slot];
+        if (!raw.alloc(at[1] - at[0] + L->plan.U_bytes[kSolid])) return no_host_memory(L);
+        if (raw.bytes)
+            KLB_CUDA(L, cudaMemcpyAsync(raw.p.get(), dev(L, at[0]), raw.bytes, cudaMemcpyDeviceToHost, L->stream));
+        klb_status st = sync(L);
+        guard.done = true;
+        if (st != KLB_OK) return st;
+        for (int s = 0; s < 3; ++s) {
+            const int c = cls_of(s);
+            const size_t ns = g.slot_row[c].size(), a0 = s == 2 ? 3 : 0;
+            auto put = [&](auto *U) {
+                rows_to_box(L, c, 3, Uo[t] + s * 3 * ncell, [&, U, ns, a0, c](size_t a, size_t r, double *o) {
+                    const int q = g.info[c][r].slot;
+                    if (q < 0) {
+                        std::memset(o, 0, nx * sizeof(double));
+                        return;
                     }
-                }
-            }
+                    const auto *v = U + ((a0 + a) * ns + (size_t)q) * nxp;
+                    for (size_t x = 0; x < nx; ++x) o[x] = (double)v[x];
+                });
+            };
+            const char *U = raw.p.get() + (at[c] - at[0]);
+            if (arith_size(L) == 8)
+                put(reinterpret_cast<const double *>(U));
+            else
+                put(reinterpret_cast<const float *>(U));
         }
     }
-    (void)ps;
     return KLB_OK;
 }
 
@@ -736,110 +887,118 @@ klb_status klb_set_state(klb_lattice *L, const double *gin, const double *U1, co
     if (!L || !gin || !U1 || !U2) return fail(L, KLB_EINVAL, "null argument");
     if (step < 0) return fail(L, KLB_EINVAL, "step must be >= 0");
     const Geometry &g = L->geo;
-    const size_t ts = arith_size(L), ncell = (size_t)g.nx * g.ny * g.nz, nxp = g.nxp;
-    const int Q = g.Q;
+    const size_t ncell = (size_t)g.nx * g.ny * g.nz, nxp = g.nxp, nx = g.nx;
+    const int Q = g.Q, storage = L->desc.storage;
     const bool red = reduced(L);
-    const double scale = L->desc.storage == KLB_FP16_DEV ? kFp16Scale : 1.0;
+    const float scale = storage == KLB_FP16_DEV ? kFp16Scale : 1.0f;
     auto sat = [](float v, float m) { return v > m ? m : (v < -m ? -m : v); };  // NaN passes
-    auto put = [&](std::vector<char> &raw, size_t k, double v) {
-        switch (L->desc.storage) {
-        case KLB_FP64:
-            ((double *)raw.data())[k] = v;
-            break;
-        case KLB_FP32:
-            ((float *)raw.data())[k] = (float)v;
-            break;
-        case KLB_FP16_DEV:  // saturating, as the device encode
-            ((__half *)raw.data())[k] = __float2half_rn(sat((float)v, 65504.0f));
-            break;
-        default:
-            ((__nv_bfloat16 *)raw.data())[k] = __float2bfloat16_rn(sat((float)v, 3.38953139e38f));
-            break;
-        }
-    };
-    auto wr = [&](std::vector<char> &raw, size_t k, double v) {
-        if (ts == 8)
-            ((double *)raw.data())[k] = v;
-        else
-            ((float *)raw.data())[k] = (float)v;
-    };
     KLB_CUDA(L, cudaStreamSynchronize(L->stream));
-    L->st.cur = 0;
-    L->st.step = step;
-    L->st.since_reset = 0;
-    L->st.gen_buf[0] = L->st.gen_buf[1] = 0;
-    L->st.refresh_pending = false;
-    std::vector<float> enc[3];
+    reset_state(L, step);
+    std::vector<float> enc[3], dec[3];
+    HostBuf pops, Us[2];
+    StreamGuard guard{L->stream};
+    const MemoryPlan &p = L->plan;
+    if (!pops.alloc(pops_bytes(L))) return no_host_memory(L);
     for (int s = 0; s < 3; ++s) {
         const int c = cls_of(s);
         const size_t nr = g.rows[c].size();
-        if (red) {
-            // Reference of each (row, direction): the x-average of the state.
-            enc[s].assign(nr * kRefStride, 0.f);
-            for (int i = 0; i < Q; ++i)
-                for (size_t r = 0; r < nr; ++r) {
-                    double sum = 0.0;
-                    for (int x = 0; x < g.nx; ++x)
-                        sum += gin[((size_t)s * Q + i) * ncell + x + (size_t)g.nx * g.rows[c][r]];
-                    enc[s][r * kRefStride + i] = (float)(sum / g.nx);
+        if (red) enc[s].assign(nr * kRefStride, 0.f);
+        auto take = [&](auto *pop) {
+            using V = std::decay_t<decltype(*pop)>;
+            host_parallel((size_t)Q * nr, (size_t)Q * nr * nx * sizeof(double), [&, pop, nr, s, c](size_t k0, size_t k1) {
+                for (size_t k = k0; k < k1; ++k) {
+                    const size_t i = k / nr, r = k - i * nr;
+                    const double *in = gin + ((size_t)s * Q + i) * ncell + nx * g.rows[c][r];
+                    V *o = pop + k * nxp;
+                    std::memset((void *)(o + nx), 0, (nxp - nx) * sizeof(V));
+                    if constexpr (std::is_same_v<V, __half> || std::is_same_v<V, __nv_bfloat16>) {
+                        // Reference of each (row, direction): the x-average of the state.
+                        double sum = 0.0;
+                        for (size_t x = 0; x < nx; ++x) sum += in[x];
+                        const float ref = (float)(sum / g.nx);
+                        enc[s][r * kRefStride + i] = ref;
+                        for (size_t x = 0; x < nx; ++x) {
+                            const float v = ((float)in[x] - ref) * scale;  // saturating, as the device encode
+                            if constexpr (std::is_same_v<V, __half>)
+                                o[x] = __float2half_rn(sat(v, 65504.0f));
+                            else
+                                o[x] = __float2bfloat16_rn(sat(v, 3.38953139e38f));
+                        }
+                    } else {
+                        for (size_t x = 0; x < nx; ++x) o[x] = (V)in[x];
+                    }
                 }
+            });
+        };
+        char *pop = pops.p.get() + (p.pop[0][s] - p.pop[0][0]);
+        switch (storage) {
+        case KLB_FP64:
+            take(reinterpret_cast<double *>(pop));
+            break;
+        case KLB_FP32:
+            take(reinterpret_cast<float *>(pop));
+            break;
+        case KLB_FP16_DEV:
+            take(reinterpret_cast<__half *>(pop));
+            break;
+        default:
+            take(reinterpret_cast<__nv_bfloat16 *>(pop));
+            break;
         }
-        std::vector<char> raw(L->plan.pop_bytes[s], 0);
-        for (int i = 0; i < Q; ++i)
-            for (size_t r = 0; r < nr; ++r) {
-                const float ref = red ? enc[s][r * kRefStride + i] : 0.f;
-                for (int x = 0; x < g.nx; ++x) {
-                    const double v = gin[((size_t)s * Q + i) * ncell + x + (size_t)g.nx * g.rows[c][r]];
-                    put(raw, (i * nr + r) * nxp + x, red ? ((float)v - ref) * (float)scale : v);
-                }
-            }
-        for (int b = 0; b < 2; ++b)
-            KLB_CUDA(L, cudaMemcpy(dev(L, L->plan.pop[b][s]), raw.data(), raw.size(),
-                                   cudaMemcpyHostToDevice));
     }
+    KLB_CUDA(L, cudaMemcpyAsync(dev(L, p.pop[0][0]), pops.p.get(), pops.bytes, cudaMemcpyHostToDevice, L->stream));
+    KLB_CUDA(L, cudaMemcpyAsync(dev(L, p.pop[1][0]), dev(L, p.pop[0][0]), pops.bytes, cudaMemcpyDeviceToDevice, L->stream));
     if (red) {
         for (int s = 0; s < 3; ++s) {
             const int c = cls_of(s);
             const size_t nr = g.rows[c].size();
-            std::vector<float> dec(nr * kRefStride, 0.f);
+            dec[s].assign(nr * kRefStride, 0.f);
             for (size_t r = 0; r < nr; ++r)
                 for (int i = 0; i < Q; ++i) {
                     const long q = g.info[c][r].src[i] / (g.nxp / kRowAlign);  // sdir * nr + srow
                     const long sdir = q / (long)nr, srow = q - sdir * (long)nr;
-                    dec[r * kRefStride + i] = enc[s][srow * kRefStride + sdir];
+                    dec[s][r * kRefStride + i] = enc[s][srow * kRefStride + sdir];
                 }
-            KLB_CUDA(L, cudaMemcpy(dev(L, L->plan.ref_enc[0][s]), enc[s].data(), L->plan.ref_bytes[s],
-                                   cudaMemcpyHostToDevice));
-            KLB_CUDA(L, cudaMemcpy(dev(L, L->plan.ref_dec[0][s]), dec.data(), L->plan.ref_bytes[s],
-                                   cudaMemcpyHostToDevice));
+            KLB_CUDA(L, cudaMemcpyAsync(dev(L, L->plan.ref_enc[0][s]), enc[s].data(), L->plan.ref_bytes[s],
+                                        cudaMemcpyHostToDevice, L->stream));
+            KLB_CUDA(L, cudaMemcpyAsync(dev(L, L->plan.ref_dec[0][s]), dec[s].data(), L->plan.ref_bytes[s],
+                                        cudaMemcpyHostToDevice, L->stream));
         }
     }
-    const double *Ui[3] = {U1, U2, U2};  // u(n-1), u(n-2); u(n-3) unknown: reuse u(n-2)
-    for (int t = 0; t < 3; ++t) {
-        const int slot = slot_of(step - 1 - t);
+    const double *Ui[2] = {U1, U2};  // u(n-1), u(n-2)
+    for (int t = 0; t < 2; ++t) {
+        const size_t *at = p.U[slot_of(step - 1 - t)], n = at[1] - at[0] + p.U_bytes[kSolid];
+        if (!Us[t].alloc(n)) return no_host_memory(L);
         for (int c = 0; c < 2; ++c) {
             const size_t ns = g.slot_row[c].size();
             if (!ns) continue;
-            std::vector<char> raw(L->plan.U_bytes[c], 0);
-            for (size_t q = 0; q < ns; ++q) {
-                const size_t cs = g.rows[c][g.slot_row[c][q]];
-                for (int x = 0; x < g.nx; ++x) {
-                    const size_t cell = x + (size_t)g.nx * cs;
-                    for (int a = 0; a < 3; ++a) {
-                        if (c == kFluid) {
-                            wr(raw, (a * ns + q) * nxp + x, Ui[t][a * ncell + cell]);
-                        } else {
-                            wr(raw, (a * ns + q) * nxp + x, Ui[t][(3 + a) * ncell + cell]);
-                            wr(raw, ((a + 3) * ns + q) * nxp + x, Ui[t][(6 + a) * ncell + cell]);
-                        }
+            auto take = [&](auto *U) {
+                using V = std::decay_t<decltype(*U)>;
+                const size_t na = c == kFluid ? 3 : 6, b0 = c == kFluid ? 0 : 3;  // component planes, first box plane
+                host_parallel(na * ns, na * ns * nx * sizeof(double), [&, U, ns, b0, c, t](size_t k0, size_t k1) {
+                    for (size_t k = k0; k < k1; ++k) {
+                        const size_t a = k / ns, q = k - a * ns;
+                        const double *in = Ui[t] + (b0 + a) * ncell + nx * g.rows[c][g.slot_row[c][q]];
+                        V *o = U + k * nxp;
+                        for (size_t x = 0; x < nx; ++x) o[x] = (V)in[x];
+                        for (size_t x = nx; x < nxp; ++x) o[x] = V(0);
                     }
-                }
-            }
-            KLB_CUDA(L, cudaMemcpy(dev(L, L->plan.U[slot][c]), raw.data(), raw.size(),
-                                   cudaMemcpyHostToDevice));
+                });
+            };
+            char *U = Us[t].p.get() + (at[c] - at[0]);
+            if (arith_size(L) == 8)
+                take(reinterpret_cast<double *>(U));
+            else
+                take(reinterpret_cast<float *>(U));
         }
+        if (n) KLB_CUDA(L, cudaMemcpyAsync(dev(L, at[0]), Us[t].p.get(), n, cudaMemcpyHostToDevice, L->stream));
+        // u(n-3) unknown: reuse u(n-2)
+        if (n && t == 1)
+            KLB_CUDA(L, cudaMemcpyAsync(dev(L, p.U[slot_of(step - 3)][0]), dev(L, at[0]), n, cudaMemcpyDeviceToDevice,
+                                        L->stream));
     }
-    return KLB_OK;
+    guard.done = true;
+    return sync(L);
 }
 
 int64_t klb_get_step(const klb_lattice *L) { return L ? L->st.step : -1; }

@@ -230,13 +230,39 @@ bool build_geometry(const klb_desc &d, Geometry &g, std::string &err)
     //     when the upstream cell or a blocked neighbour is void (outer wall);
     //     else free-slip (specular): reverse the blocked components, pull
     //     from the cell shifted back along the unblocked axes.
+    // Rows whose eight neighbours all carry the class (most of them) take
+    // plain streaming without further tests.
     for (int cls = 0; cls < 2; ++cls) {
         const int ct = class_cell_type(cls);
         const int nr = (int)g.rows[cls].size();
+        const int unit = g.nxp / kRowAlign;
+        uint32_t xm_all = 0, xp_all = 0;
+        int shift_cs[19];
+        for (int i = 0; i < g.Q; ++i) {
+            if (v.c[i][0] == 1) xm_all |= 1u << i;   // source at x - 1
+            if (v.c[i][0] == -1) xp_all |= 1u << i;  // source at x + 1
+            shift_cs[i] = -v.c[i][1] - d.ny * v.c[i][2];
+        }
+        // Every population must be pulled exactly once (mass conservation).
+        std::vector<uint8_t> used((size_t)g.Q * nr, 0);
         for (int r = 0; r < nr; ++r) {
             RowInfo &ri = g.info[cls][r];
             int k = g.rows[cls][r], y = k % d.ny, z = k / d.ny;
+            bool plain = y > 0 && y < d.ny - 1 && (g.Q == 9 || (z > 0 && z < d.nz - 1));
+            for (int dz = g.Q == 9 ? 0 : -1; plain && dz <= (g.Q == 9 ? 0 : 1); ++dz)
+                for (int dy = -1; dy <= 1; ++dy) plain = plain && g.cs_type[k + dy + d.ny * dz] == ct;
+            if (plain) {
+                ri.xm = xm_all;
+                ri.xp = xp_all;
+            }
             for (int i = 0; i < g.Q; ++i) {
+                if (plain) {
+                    const int srow = g.row_of_cs[cls][k + shift_cs[i]];
+                    const long e = (long)i * nr + srow;
+                    ri.src[i] = (int32_t)(e * unit);
+                    if (used[e]++) return err = "boundary rule is not a permutation for this geometry", false;
+                    continue;
+                }
                 const int cx = v.c[i][0], cy = v.c[i][1], cz = v.c[i][2];
                 int sy = y - cy, sz = z - cz, sdir = i, sx = cx;
                 int tu = cs.type(y - cy, z - cz);
@@ -258,19 +284,14 @@ bool build_geometry(const klb_desc &d, Geometry &g, std::string &err)
                 }
                 int srow = g.row_of_cs[cls][cs.index(sy, sz)];
                 if (srow < 0 || sdir < 0) return err = "internal: streaming source off the species", false;
-                ri.src[i] = (int32_t)(((long)sdir * nr + srow) * (g.nxp / kRowAlign));
+                const long e = (long)sdir * nr + srow;
+                ri.src[i] = (int32_t)(e * unit);
                 if (sx == 1) ri.xm |= 1u << i;   // source at x - 1
                 if (sx == -1) ri.xp |= 1u << i;  // source at x + 1
                 if (cx != 0 && sx == 0) ri.flags |= kXBounce;
-            }
-        }
-        // Every population must be pulled exactly once (mass conservation).
-        std::vector<uint8_t> used((size_t)g.Q * nr, 0);
-        for (int r = 0; r < nr; ++r)
-            for (int i = 0; i < g.Q; ++i) {
-                long e = g.info[cls][r].src[i] / (g.nxp / kRowAlign);
                 if (used[e]++) return err = "boundary rule is not a permutation for this geometry", false;
             }
+        }
     }
 
     // ---- slip-fit and wall-row flags of fluid rows
@@ -332,6 +353,7 @@ MemoryPlan plan_memory(const Geometry &g, int storage)
     p.nchunk = (g.nx + p.bx - 1) / p.bx;
     p.nblocks_w = (int)nr[kFluid] * p.nchunk;
     p.nblocks_s = (int)nr[kSolid] * p.nchunk;
+    p.ep = false;
     if (storage == KLB_FP64) {
         p.sbx = fp64_split(g.nx, (int)nr[kFluid], (int)nr[kSolid]) ? 32 : p.bx;
         p.static_blocks = p.nblocks_w + p.nblocks_s;
@@ -354,7 +376,6 @@ MemoryPlan plan_memory(const Geometry &g, int storage)
     }
     p.partials = take(sizeof(double) * kNumSums * std::max((size_t)(p.nblocks_w + p.nblocks_s), (size_t)p.oblocks));
     p.sums = take(sizeof(double) * kNumSums + sizeof(unsigned));
-    p.ep = false;
     p.obs_done = p.sums + sizeof(double) * kNumSums;
     p.field_bytes = ts * 4 * (nr[kFluid] + 2 * nr[kSolid]) * g.nxp;
     p.field = take(p.field_bytes);
