@@ -18,7 +18,8 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(BUILD, "libklb.so")
-SOURCES = ["klb_kernels_q19.cu", "klb_kernels_q19_16.cu", "klb_kernels_q9.cu", "klb_kernels.cu", "klb_geometry.cpp",
+SOURCES = ["klb_batch_q19_16.cu", "klb_kernels_q19_16.cu", "klb_batch_q19.cu", "klb_kernels_q19.cu",
+           "klb_batch_q9.cu", "klb_kernels_q9.cu", "klb_kernels.cu", "klb_geometry.cpp",
            "klb_api.cpp", "klb_static.cu", "klb_server.cpp"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

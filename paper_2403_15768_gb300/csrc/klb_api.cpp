@@ -1044,6 +1044,8 @@ struct klb_batch {
     int nblocks = 0;
     bool ep = false;
     size_t args_size = 0, table_off = 0, prefix_off = 0, reps_off = 0;
+    std::vector<char> table;      // host copies of the argument tables and the block prefix
+    std::vector<int> prefix;
     std::vector<StepPlan> plans;  // per (phase, member)
     std::vector<char> acc;        // per phase: some member accumulates x-sums
     std::vector<int64_t> base_step;  // members' steps at phase 0
@@ -1097,8 +1099,10 @@ void destroy_graph(klb_batch *B)
 klb_status build_tables(klb_batch *B, int width)
 {
     const int n = (int)B->mem.size(), P = B->period;
-    std::vector<char> host((size_t)P * n * B->args_size);
-    std::vector<int> prefix(n + 1, 0);
+    std::vector<char> &host = B->table;
+    std::vector<int> &prefix = B->prefix;
+    host.assign((size_t)P * n * B->args_size, 0);
+    prefix.assign(n + 1, 0);
     B->plans.assign((size_t)P * n, StepPlan{0, false, false});
     B->acc.assign(P, 0);
     size_t all_bytes = 0;
@@ -1166,9 +1170,10 @@ cudaError_t launch_phase(klb_batch *B, int k)
         L->stream = keep;
         if (e != cudaSuccess) return e;
     }
-    const char *table = B->base + B->table_off + (size_t)k * n * B->args_size;
-    cudaError_t e = launch_batch(B->Q, B->storage, table, (const int *)(B->base + B->prefix_off), (int)n,
-                                 B->nblocks, B->width, B->acc[k] != 0, B->ep, B->stream);
+    const size_t at = (size_t)k * n * B->args_size;
+    const BatchLaunch b{B->table.data() + at, B->base + B->table_off + at, B->prefix.data(),
+                        (const int *)(B->base + B->prefix_off), (int)n, B->width, B->acc[k] != 0, B->ep};
+    cudaError_t e = launch_batch(B->Q, B->storage, b, B->stream);
     if (e == cudaSuccess && k == B->period - 1) e = launch_count_period((uint32_t *)(B->base + B->reps_off), B->stream);
     return e;
 }

@@ -243,10 +243,23 @@ cudaError_t launch_ref(int Q, int storage, const void *args, float *const enc[3]
 cudaError_t launch_finalize(const double *partials, int nblocks, double *sums, cudaStream_t s);
 // One more period completed by a batch (StepArgs::step_reps).
 cudaError_t launch_count_period(uint32_t *reps, cudaStream_t s);
-// One step of many lattices in one launch: table[l] holds the arguments of
-// lattice l, prefix[l] its first block (prefix[n] = total blocks).
-cudaError_t launch_batch(int Q, int storage, const void *table, const int *prefix, int n,
-                         int nblocks, int bx, bool acc, bool ep, cudaStream_t s);
+// One step of many lattices: argument records (host and device copies) and
+// first block of each lattice (prefix[n] = total blocks).  Up to
+// kBatchParams records go as kernel parameters (32 KB hold 56 of FP64); more
+// lattices take several such launches if the step has at least kGroupBlocks
+// blocks, else one launch over the device table: a launch waits for the one
+// before it.  One launch over the table -> several: 64 channels of a sweep
+// FP32 2410 -> 2310 us, FP16 2305 -> 2162; 100 pipes of R 6-9, nx 8 (8800
+// blocks) FP32 84.7 -> 82.8, FP16 127.2 -> 125.9.
+constexpr int kBatchParams = 56;
+constexpr int kGroupBlocks = 4000;
+struct BatchLaunch {
+    const void *table, *dev_table;
+    const int *prefix, *dev_prefix;
+    int n, width;
+    bool acc, ep;
+};
+cudaError_t launch_batch(int Q, int storage, const BatchLaunch &b, cudaStream_t s);
 
 // Device bytes of the argument tables of a batch of n lattices with this
 // storage (the layout klb_batch_create uses).

@@ -11,16 +11,14 @@ cudaError_t launch_q19(int storage, const void *args, int mode, int nblocks, int
 cudaError_t launch_ref_q9(const void *args, float *const enc[3], float *const dec[3], cudaStream_t s);
 cudaError_t launch_ref_q19(const void *args, float *const enc[3], float *const dec[3], cudaStream_t s);
 
-cudaError_t launch_batch_q9(int storage, const void *table, const int *prefix, int n, int nblocks,
-                          int bx, bool acc, bool ep, cudaStream_t s);
-cudaError_t launch_batch_q19(int storage, const void *table, const int *prefix, int n, int nblocks,
-                           int bx, bool acc, bool ep, cudaStream_t s);
+cudaError_t launch_batch_q9(int storage, const BatchLaunch &b, cudaStream_t s);
+cudaError_t launch_batch_q19(int storage, const BatchLaunch &b, cudaStream_t s);
+cudaError_t launch_batch_q19_16(int storage, const BatchLaunch &b, cudaStream_t s);
 
-cudaError_t launch_batch(int Q, int storage, const void *table, const int *prefix, int n,
-                         int nblocks, int bx, bool acc, bool ep, cudaStream_t s)
+cudaError_t launch_batch(int Q, int storage, const BatchLaunch &b, cudaStream_t s)
 {
-    return Q == 9 ? launch_batch_q9(storage, table, prefix, n, nblocks, bx, acc, ep, s)
-                  : launch_batch_q19(storage, table, prefix, n, nblocks, bx, acc, ep, s);
+    if (Q == 9) return launch_batch_q9(storage, b, s);
+    return reduced_storage(storage) ? launch_batch_q19_16(storage, b, s) : launch_batch_q19(storage, b, s);
 }
 
 cudaError_t launch(int Q, int storage, const void *args, int mode, int nblocks, int bx,

@@ -22,17 +22,4 @@ cudaError_t launch_ref_q19(const void *args, float *const enc[3], float *const d
     return launch_ref_q<19, float>(args, enc, dec, s);
 }
 
-cudaError_t launch_batch_q19_16(int storage, const void *table, const int *prefix, int n, int nblocks,
-                                int bx, bool acc, bool ep, cudaStream_t s)
-{
-    switch (storage) {
-    case KLB_FP16_DEV:
-        return launch_batch_q<19, float, __half>(table, prefix, n, nblocks, bx, acc, ep, s);
-    case KLB_BF16_DEV:
-        return launch_batch_q<19, float, __nv_bfloat16>(table, prefix, n, nblocks, bx, acc, ep, s);
-    default:
-        return cudaErrorInvalidValue;
-    }
-}
-
 }  // namespace klb
