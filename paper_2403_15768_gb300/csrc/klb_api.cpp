@@ -166,6 +166,7 @@ void fill_args_at(const klb_lattice *L, const HostState &st, int sbx, bool ep, s
     a.step_lo = (uint32_t)((uint64_t)n & 0xffffffffu);
     a.step_hi = (uint32_t)((uint64_t)n >> 32);
     a.bounds_err = (unsigned *)dev(L, p.bounds);
+    for (int s = 0; s < 3; ++s) a.ck[s] = collide_k(g.Q, (float)a.om[s]);
     a.ahead = step_ahead(g.Q, d.storage, g.nxp, all_bytes);
 }
 

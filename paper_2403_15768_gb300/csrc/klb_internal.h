@@ -177,6 +177,31 @@ inline int step_ahead(int Q, int storage, int nxp, size_t all_bytes)
     return (int)((ahead + row - 1) / row);
 }
 
+// Collision constants of one relaxation rate om (fo = 1 - om/2) per weight
+// class (rest, axis, edge directions), as the pairs that the packed
+// instructions take: from the kernel's parameters they need no moves and no
+// arithmetic in the kernel (512x128x128 FP16 108.1 -> 106.0 us, 768x192x192
+// FP16 344.1 -> 338.7, 12-channel sweep FP16 410 -> 401, FP32 456 -> 453).
+struct CollideK {
+    float2 om1, omw[3], fow[3], tow[3], tfw[3];  // 1 - om, om w, fo w, 3 om w, 3 fo w
+};
+inline __host__ __device__ CollideK collide_k(int Q, float om)
+{
+    const float w[3] = {Q == 19 ? float(1.0 / 3.0) : float(4.0 / 9.0), Q == 19 ? float(1.0 / 18.0) : float(1.0 / 9.0),
+                        float(1.0 / 36.0)};
+    const float om1 = 1.f - om, fo = 1.f - 0.5f * om;
+    CollideK c;
+    c.om1 = make_float2(om1, om1);
+    for (int k = 0; k < 3; ++k) {
+        const float v[4] = {om * w[k], fo * w[k], 3.f * om * w[k], 3.f * fo * w[k]};
+        c.omw[k] = make_float2(v[0], v[0]);
+        c.fow[k] = make_float2(v[1], v[1]);
+        c.tow[k] = make_float2(v[2], v[2]);
+        c.tfw[k] = make_float2(v[3], v[3]);
+    }
+    return c;
+}
+
 // Kernel arguments.  T is the arithmetic type (float or double); the
 // populations are stored as T, or as FP16/BF16 against per-row references.
 template <typename T>
@@ -219,6 +244,7 @@ struct alignas(16) StepArgs {
     const uint32_t *step_reps;
     int step_period;
     int ahead;             // rows ahead whose populations the step asks L2 for (step_ahead; 0: none)
+    CollideK ck[3];        // FP32 arithmetic: collision constants per species
     unsigned *bounds_err;  // debug builds: first out-of-range index site
 };
 
@@ -245,13 +271,13 @@ cudaError_t launch_finalize(const double *partials, int nblocks, double *sums, c
 cudaError_t launch_count_period(uint32_t *reps, cudaStream_t s);
 // One step of many lattices: argument records (host and device copies) and
 // first block of each lattice (prefix[n] = total blocks).  Up to
-// kBatchParams records go as kernel parameters (32 KB hold 56 of FP64); more
+// kBatchParams records go as kernel parameters (32 KB in all); more
 // lattices take several such launches if the step has at least kGroupBlocks
 // blocks, else one launch over the device table: a launch waits for the one
 // before it.  One launch over the table -> several: 64 channels of a sweep
 // FP32 2410 -> 2310 us, FP16 2305 -> 2162; 100 pipes of R 6-9, nx 8 (8800
 // blocks) FP32 84.7 -> 82.8, FP16 127.2 -> 125.9.
-constexpr int kBatchParams = 56;
+constexpr int kBatchParams = 36;
 constexpr int kGroupBlocks = 4000;
 struct BatchLaunch {
     const void *table, *dev_table;

@@ -335,7 +335,7 @@ __device__ __forceinline__ uint32_t dither_seed(uint32_t cs, uint32_t n, int s)
 // differences to nearest anyway and keeps the plain fix-up.
 template <int Q, bool FIX = true, bool DITHER = false>
 __device__ __forceinline__ void collide2(float2 g[Q], const Cell2 &c, const float2 j[3], float rho0,
-                                         float om, float q = 1.f, uint32_t sd = 0u)
+                                         float q, uint32_t sd, const CollideK &K)
 {
     const float2 rho = add2(b2(rho0), c.drho);
     const float2 uu = fma2(c.u[2], c.u[2], fma2(c.u[1], c.u[1], mul2(c.u[0], c.u[0])));
@@ -343,40 +343,38 @@ __device__ __forceinline__ void collide2(float2 g[Q], const Cell2 &c, const floa
     const float2 e0 = fma2(mul2(b2(-1.5f * q), rho), uu, c.drho);
     const float2 r45 = mul2(b2(4.5f * q), rho);
     const float2 m3uF = mul2(b2(-3.f * q), uF);
-    const float om1 = 1.f - om, fo = 1.f - 0.5f * om;
     constexpr bool DIFF = FIX && DITHER;
     float2 dm = b2(0.f), dj[3] = {b2(0.f), b2(0.f), b2(0.f)};  // Sum (g - g*), Sum c (g - g*)
     {
-        const float w = float(wt<Q>(0));
         const float2 g0 = g[0];
-        g[0] = fma2(b2(om1), g[0], fma2(b2(om * w), e0, mul2(b2(fo * w), m3uF)));
+        g[0] = fma2(K.om1, g[0], fma2(K.omw[0], e0, mul2(K.fow[0], m3uF)));
         if constexpr (DIFF) dm = sub2(g0, g[0]);
     }
 #pragma unroll
     for (int i = 1; i < Q; ++i) {
         if (opp<Q>(i) < i) continue;
         const int ib = opp<Q>(i);
-        const float w = float(wt<Q>(i));
+        const int k = (cx<Q>(i) != 0) + (cy<Q>(i) != 0) + (cz<Q>(i) != 0);  // weight class
         const float2 cu = cdot2<Q>(i, c.u);
         const float2 cF = cdot2<Q>(i, c.F);
         // even parts: e0 + 4.5 rho cu^2 and -3 u.F + 9 cu cF
         const float2 se = fma2(r45, mul2(cu, cu), e0);
         const float2 sf = fma2(b2(9.f * q), mul2(cu, cF), m3uF);
-        const float2 S = fma2(b2(om * w), se, mul2(b2(fo * w), sf));
+        const float2 S = fma2(K.omw[k], se, mul2(K.fow[k], sf));
         // odd parts: 3 rho cu and 3 cF
-        const float2 A = fma2(mul2(b2(3.f * om * w), rho), cu, mul2(b2(3.f * fo * w), cF));
+        const float2 A = fma2(mul2(K.tow[k], rho), cu, mul2(K.tfw[k], cF));
         const float2 gi = g[i], gb = g[ib];
-        g[i] = fma2(b2(om1), gi, add2(S, A));
-        g[ib] = fma2(b2(om1), gb, sub2(S, A));
+        g[i] = fma2(K.om1, gi, add2(S, A));
+        g[ib] = fma2(K.om1, gb, sub2(S, A));
         if constexpr (DIFF) {
             const float2 di = sub2(gi, g[i]), db = sub2(gb, g[ib]);
             dm = add2(dm, add2(di, db));
             const float2 dd = sub2(di, db);
             const int cc[3] = {cx<Q>(i), cy<Q>(i), cz<Q>(i)};
 #pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                if (cc[k] > 0) dj[k] = add2(dj[k], dd);
-                if (cc[k] < 0) dj[k] = sub2(dj[k], dd);
+            for (int a = 0; a < 3; ++a) {
+                if (cc[a] > 0) dj[a] = add2(dj[a], dd);
+                if (cc[a] < 0) dj[a] = sub2(dj[a], dd);
             }
         }
     }
@@ -705,6 +703,14 @@ __device__ __forceinline__ void step_body2(const StepArgs<float> &p, int b)
     constexpr bool DITHER = !Storage<S>::kRef;
     const uint32_t n_step = p.step_lo + (p.step_reps ? *p.step_reps * (uint32_t)p.step_period : 0u);
 
+    // (with thermal noise, formed in the kernel: there they cost nothing that
+    // counts, and the compiler rounds the noise as it did)
+    auto consts = [&](int s) -> CollideK {
+        if constexpr (NOISE)
+            return collide_k(Q, p.om[s]);
+        else
+            return p.ck[s];
+    };
     if (water) {
         float2 g[Q], j[3];
         Cell2 c;
@@ -715,7 +721,7 @@ __device__ __forceinline__ void step_body2(const StepArgs<float> &p, int b)
             const int ns = p.n_slots[kFluid];
             for (int a = 0; a < 3; ++a) store_u2(p.U0[kFluid] + (a * ns + q5.y) * nxp + X.x0, c.u[a]);
         }
-        collide2<Q, true, DITHER>(g, c, j, p.rho0, p.om[0], 1.f, dither_seed((uint32_t)q7.y, n_step, 0));
+        collide2<Q, true, DITHER>(g, c, j, p.rho0, 1.f, dither_seed((uint32_t)q7.y, n_step, 0), consts(0));
         if constexpr (NOISE) {
             const uint32_t cell = (uint32_t)X.x0 + (uint32_t)p.nx * (uint32_t)q7.y;
             thermal_noise<Q, float>(p, cell, [&](int i, float v) { g[i].x += v; });
@@ -803,7 +809,7 @@ __device__ __forceinline__ void step_body2(const StepArgs<float> &p, int b)
         }
     }
     const int stride = p.n_rows[kSolid] * nxp, base = row * nxp + X.x0;
-    collide2<Q, true, DITHER>(ge, ce, je, p.rho0, p.om[1], 1.f, dither_seed((uint32_t)q7.y, n_step, 1));
+    collide2<Q, true, DITHER>(ge, ce, je, p.rho0, 1.f, dither_seed((uint32_t)q7.y, n_step, 1), consts(1));
     if (live)
         store_pair<Q, S>(ge, static_cast<S *>(p.out[1]), stride, base, ref_row<float, S>(p.enc_out[1], row), sc);
     float acc[ACC ? 2 * Q : 1];
@@ -813,7 +819,7 @@ __device__ __forceinline__ void step_body2(const StepArgs<float> &p, int b)
     }
     pull_row2<Q, S>(static_cast<const S *>(p.in[2]), src, xm, xp, xbounce, X,
                     ref_row<float, S>(p.dec_in[2], row), inv, gp);
-    collide2<Q, true, DITHER>(gp, cp, jp, p.rho0, p.om[2], p.q_p, dither_seed((uint32_t)q7.y, n_step, 2));
+    collide2<Q, true, DITHER>(gp, cp, jp, p.rho0, p.q_p, dither_seed((uint32_t)q7.y, n_step, 2), consts(2));
     if (live)
         store_pair<Q, S>(gp, static_cast<S *>(p.out[2]), stride, base, ref_row<float, S>(p.enc_out[2], row), sc);
     if constexpr (ACC) {
