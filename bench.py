@@ -410,9 +410,9 @@ def run(args):
                      "peak_source": peak_kind,
                      "bytes_per_launch": bytes_per_launch, "launch_ms": step_kernel_ms},
         "e2e": {"value": e2e_value, "unit": "MLUPS", "h2d_bytes_per_step": 40,
-                "d2h_bytes_per_step": 144},
+                "d2h_bytes_per_step": 120},
         "species_cell_updates": {"value": value * species_cells / sites, "unit": "M species-cells/s"},
-        "gpu_launches": args.steps * (LATTICE_STEPS_PER_STEP + 2),
+        "gpu_launches": args.steps * (LATTICE_STEPS_PER_STEP + 1),
         "clocks": clk.summary(),
         "observables": {"flow_rate": obs["flow_rate"], "slip_length": obs["slip_length"],
                         "step": obs["step"], "e2e_step": obs_e2e["step"]},
@@ -518,11 +518,12 @@ def run_sweep(args):
                    "l2": f"working set {sum(l.nbytes for l in lats) / 1e9:.1f} GB > 129 MB L2, no flush needed"},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": None,
-                     "kernel": f"k_step_batch<19,float,{storage}>", "peak_source": peak_kind,
+                     "kernel": f"k_step_group<19,float,{storage}>", "peak_source": peak_kind,
                      "bytes_per_launch": bytes_per_launch, "launch_ms": step_ms},
         "e2e": {"value": updates / (e2e_ms * 1e-3) / 1e6, "unit": "MLUPS",
-                "h2d_bytes_per_step": 40 * len(lats), "d2h_bytes_per_step": 144 * len(lats)},
-        "gpu_launches": args.steps * (SWEEP_STEPS + 2 * len(lats) +
+                "h2d_bytes_per_step": 40 * len(lats), "d2h_bytes_per_step": 120 * len(lats)},
+        # batched steps (36 lattices per launch), one observation and the reference refreshes per lattice
+        "gpu_launches": args.steps * (SWEEP_STEPS * -(-len(lats) // 36) + len(lats) +
                                       (2 * len(lats) * SWEEP_STEPS // 32 if storage != "fp32" else 0)),
         "clocks": clk.summary(),
         "observables": {"flow_rate_first3": [o["flow_rate"] for o in obs[:3]],

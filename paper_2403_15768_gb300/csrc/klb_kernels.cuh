@@ -1,5 +1,5 @@
 // CUDA kernels of the KLB step for sm_103a (templates; instantiated per
-// lattice in klb_kernels_q9.cu and klb_kernels_q19.cu).
+// lattice in klb_kernels_q*.cu and klb_batch_q*.cu).
 //
 // One fused kernel per lattice step (k_step) updates all three species
 // (Sec. 4: one population set per species, {h_i, e_i, p_i}):
@@ -11,12 +11,13 @@
 //
 // Layout: structure of arrays, per species [direction][row][x] with rows of
 // nxp elements (x fastest, rows padded to 32 elements), so every load and
-// store of a warp is a contiguous run of x.  A block covers up to 128
-// consecutive x of one row; the row table (sources, x shifts, interface
-// partners) is block-uniform.  A solid block updates the electrons and
-// phonons of its row together; the step grid puts the solid blocks first
-// (the heavier work, so that its last wave holds water blocks), the
-// observation, field and initialisation grids the water blocks first.
+// store of a warp is a contiguous run of x.  With FP32 arithmetic the step
+// and the observation give each warp 64 cells of a row, with FP64 (and in the
+// field and initialisation passes) a block covers up to 128 cells of one row;
+// the row table (sources, x shifts, interface partners) is warp-uniform.
+// Solid work updates the electrons and phonons of a cell together and comes
+// first in the step and observation grids (the heavier work, so that the last
+// wave holds water), the water first in the other grids.
 //
 // Template parameters: Q (9 or 19), T the arithmetic type (double or float)
 // and S the storage type of the populations (T itself, or __half /
@@ -27,9 +28,9 @@
 // The reference of a pulled population is that of its source row (table
 // `dec`), the reference of a stored one that of its own row (table `enc`).
 //
-// k_lattice runs the same per-cell arithmetic for the observation pass
-// (velocities of the current and previous step reduced in FP64) and the
-// field pass; k_init starts from local equilibria.
+// k_lattice runs the same per-cell arithmetic for the field pass and the FP64
+// observation pass (velocities of the current and previous step reduced in
+// FP64; FP32 arithmetic: k_observe2); k_init starts from local equilibria.
 
 #pragma once
 
@@ -793,19 +794,20 @@ __global__ void __launch_bounds__(kBlockX) k_init(const StepArgs<T> p)
 // ---------------------------------------------------------------------------
 // Step kernel.
 //
-// One block per work item (one row, up to 128 threads along x).  With FP32
-// arithmetic a thread updates two adjacent cells (klb_step_pair.cuh), in
-// FP64 one (step_body below).  Memory parallelism comes from residency: the
-// FP32-arithmetic kernel is held to 96 registers (5 blocks of 128 threads
-// per SM; a few spilled values cost less than the occupancy they buy), and
-// every thread issues its loads back to back.  The row table is read with
+// FP32 arithmetic: one warp per 64 cells of a row, two adjacent cells per
+// thread (klb_step_pair.cuh); FP64: one block per row chunk, one cell per
+// thread (step_body below).  Memory parallelism comes from residency and from
+// L2 requests for later rows: the FP32-arithmetic kernel is held to 96
+// registers (5 blocks of 128 threads per SM; at 128 and 4 blocks 512x128x128
+// takes 7% longer, at 80 and 6 blocks 2%), and every thread issues its loads
+// back to back.  The row table is read with
 // 16-byte loads (one 128-byte line per row, cached); the x shift of each
 // direction is a compile-time constant except on the few rows where an
 // x-moving population bounces back.  A solid cell streams, and takes the
 // moments of, both its electrons and phonons, then collides and stores the
 // electrons before pulling the phonons a second time (the lines are still
 // cached), so that at most Q populations are live at once.  With ACC the
-// block also writes the x-sums of its post-collision populations to p.acc
+// warp also writes the x-sums of its post-collision populations to p.acc
 // for the next reference refresh of reduced-precision storage.
 
 template <int Q, typename T, typename S>

@@ -4,7 +4,7 @@
 // scalar counterpart would be).  Used for FP32 arithmetic (FP32, FP16 and
 // BF16 storage); FP64 keeps one cell per thread.
 //
-// A thread owns the adjacent cells x0 = 2t and x0 + 1 of one row, so the
+// A thread owns two adjacent cells x0 (even) and x0 + 1 of one row, so the
 // populations of both come from one aligned 8-byte (FP32) or 4-byte (16-bit)
 // word wherever the direction does not move along x; an x-moving direction
 // pulls its two cells from x0 - 1, x0 (c_x = +1) or x0 + 1, x0 + 2
