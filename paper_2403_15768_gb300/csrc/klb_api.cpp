@@ -736,7 +736,11 @@ klb_status klb_observables_static(klb_lattice *L, klb_obs *out)
                     "observation pass needs " + std::to_string(static_blocks(L)) +
                         " blocks, more than the static scratch holds (KLB_STATIC_MAX_BLOCKS = " +
                         std::to_string(max_blocks) + ")");
-    KLB_CUDA(L, launch_observe(L, partials, sums, reinterpret_cast<unsigned *>(sums + kNumSums)));
+    // The count of finished blocks starts from 0 whatever an overlapping call
+    // (which the header asks callers to avoid) may have left.
+    unsigned *done = reinterpret_cast<unsigned *>(sums + kNumSums);
+    KLB_CUDA(L, cudaMemsetAsync(done, 0, sizeof *done, L->stream));
+    KLB_CUDA(L, launch_observe(L, partials, sums, done));
     double S[kNumSums];
     KLB_CUDA(L, cudaMemcpyAsync(S, sums, sizeof S, cudaMemcpyDeviceToHost, L->stream));
     klb_status st = sync(L);
