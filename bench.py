@@ -412,7 +412,7 @@ def run(args):
         "e2e": {"value": e2e_value, "unit": "MLUPS", "h2d_bytes_per_step": 40,
                 "d2h_bytes_per_step": 120},
         "species_cell_updates": {"value": value * species_cells / sites, "unit": "M species-cells/s"},
-        "gpu_launches": args.steps * (LATTICE_STEPS_PER_STEP + 1),
+        "gpu_launches": args.steps * (LATTICE_STEPS_PER_STEP + 2),
         "clocks": clk.summary(),
         "observables": {"flow_rate": obs["flow_rate"], "slip_length": obs["slip_length"],
                         "step": obs["step"], "e2e_step": obs_e2e["step"]},
@@ -522,8 +522,8 @@ def run_sweep(args):
                      "bytes_per_launch": bytes_per_launch, "launch_ms": step_ms},
         "e2e": {"value": updates / (e2e_ms * 1e-3) / 1e6, "unit": "MLUPS",
                 "h2d_bytes_per_step": 40 * len(lats), "d2h_bytes_per_step": 120 * len(lats)},
-        # batched steps (36 lattices per launch), one observation and the reference refreshes per lattice
-        "gpu_launches": args.steps * (SWEEP_STEPS * -(-len(lats) // 36) + len(lats) +
+        # batched steps (36 lattices per launch), one observation (two kernels) and the reference refreshes per lattice
+        "gpu_launches": args.steps * (SWEEP_STEPS * -(-len(lats) // 36) + 2 * len(lats) +
                                       (2 * len(lats) * SWEEP_STEPS // 32 if storage != "fp32" else 0)),
         "clocks": clk.summary(),
         "observables": {"flow_rate_first3": [o["flow_rate"] for o in obs[:3]],

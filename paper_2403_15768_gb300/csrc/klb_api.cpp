@@ -240,31 +240,27 @@ cudaError_t refresh_refs(const klb_lattice *L, int gen)
 
 int nblocks(const klb_lattice *L) { return L->plan.nblocks_w + L->plan.nblocks_s; }
 
-// Observation pass enqueued on the lattice's stream, its kNumSums sums in
-// `sums`: one kernel with FP32 arithmetic (`done` counts its finished
-// blocks, 0 before and after), the pass and its final reduction with FP64.
-cudaError_t launch_observe(const klb_lattice *L, double *partials, double *sums, unsigned *done)
+// Observation pass enqueued on the lattice's stream: the pass and the
+// reduction of its blocks' partial sums to the kNumSums sums.
+cudaError_t launch_observe(const klb_lattice *L, double *partials, double *sums)
 {
-    if (L->desc.storage == KLB_FP64) {
-        StepArgs<double> a;
-        fill_args(L, a);
-        a.partials = partials;
-        cudaError_t e = launch(L->geo.Q, L->desc.storage, &a, kModeObserve, nblocks(L), L->plan.bx, L->stream);
-        return e != cudaSuccess ? e : launch_finalize(partials, nblocks(L), sums, L->stream);
-    }
-    StepArgs<float> a;
-    fill_args(L, a);
-    a.partials = partials;
-    a.obs_sums = sums;
-    a.obs_done = done;
-    a.obs_solid = L->plan.oblocks_s;
-    return launch(L->geo.Q, L->desc.storage, &a, kModeObserve, L->plan.oblocks, kBlockX, L->stream);
+    const bool f64 = L->desc.storage == KLB_FP64;
+    const int blocks = f64 ? nblocks(L) : L->plan.oblocks;
+    const cudaError_t e = with_args(L, [&](void *a) {
+        if (f64) {
+            static_cast<StepArgs<double> *>(a)->partials = partials;
+        } else {
+            static_cast<StepArgs<float> *>(a)->partials = partials;
+            static_cast<StepArgs<float> *>(a)->obs_solid = L->plan.oblocks_s;
+        }
+        return launch(L->geo.Q, L->desc.storage, a, kModeObserve, blocks, f64 ? L->plan.bx : kBlockX, L->stream);
+    });
+    return e != cudaSuccess ? e : launch_finalize(partials, blocks, sums, L->stream);
 }
 
 cudaError_t launch_observe(const klb_lattice *L)
 {
-    return launch_observe(L, (double *)dev(L, L->plan.partials), (double *)dev(L, L->plan.sums),
-                          (unsigned *)dev(L, L->plan.obs_done));
+    return launch_observe(L, (double *)dev(L, L->plan.partials), (double *)dev(L, L->plan.sums));
 }
 
 // Blocks that bound the lattices klb_observables_static takes.
@@ -601,7 +597,6 @@ klb_status klb_create_lattice(const klb_desc *desc, void *dev_buf, size_t bytes,
                             sizeof(RowInfo) * L->geo.info[c].size(), cudaMemcpyHostToDevice,
                             L->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(dev(L, L->plan.bounds), 0, sizeof(unsigned), L->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(dev(L, L->plan.obs_done), 0, sizeof(unsigned), L->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(L->stream);
     if (e != cudaSuccess) {
         std::string m = std::string("uploading row tables: ") + cudaGetErrorString(e);
@@ -736,11 +731,7 @@ klb_status klb_observables_static(klb_lattice *L, klb_obs *out)
                     "observation pass needs " + std::to_string(static_blocks(L)) +
                         " blocks, more than the static scratch holds (KLB_STATIC_MAX_BLOCKS = " +
                         std::to_string(max_blocks) + ")");
-    // The count of finished blocks starts from 0 whatever an overlapping call
-    // (which the header asks callers to avoid) may have left.
-    unsigned *done = reinterpret_cast<unsigned *>(sums + kNumSums);
-    KLB_CUDA(L, cudaMemsetAsync(done, 0, sizeof *done, L->stream));
-    KLB_CUDA(L, launch_observe(L, partials, sums, done));
+    KLB_CUDA(L, launch_observe(L, partials, sums));
     double S[kNumSums];
     KLB_CUDA(L, cudaMemcpyAsync(S, sums, sizeof S, cudaMemcpyDeviceToHost, L->stream));
     klb_status st = sync(L);

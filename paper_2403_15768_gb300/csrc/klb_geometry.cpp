@@ -375,8 +375,7 @@ MemoryPlan plan_memory(const Geometry &g, int storage)
         p.oblocks = p.oblocks_s + std::min(mw, std::max(1, total - p.oblocks_s));
     }
     p.partials = take(sizeof(double) * kNumSums * std::max((size_t)(p.nblocks_w + p.nblocks_s), (size_t)p.oblocks));
-    p.sums = take(sizeof(double) * kNumSums + sizeof(unsigned));
-    p.obs_done = p.sums + sizeof(double) * kNumSums;
+    p.sums = take(sizeof(double) * kNumSums);
     p.field_bytes = ts * 4 * (nr[kFluid] + 2 * nr[kSolid]) * g.nxp;
     p.field = take(p.field_bytes);
     for (int s = 0; s < 3; ++s) p.ref_bytes[s] = 0;

@@ -89,7 +89,7 @@ struct MemoryPlan {
     size_t U[3][2];        // [time slot][row class]
     size_t U_bytes[2];
     size_t rows[2];
-    size_t partials, sums, obs_done, field;
+    size_t partials, sums, field;
     size_t field_bytes;
     size_t ref_enc[2][3], ref_dec[2][3];  // [generation][species], reduced storage only
     size_t ref_bytes[3];
@@ -224,9 +224,7 @@ struct alignas(16) StepArgs {
     T g_we, g_wp, g_ep, g_ec, g_pc;
     T q_p;                 // phonons: 1 second-order equilibrium, 0 linear (damped waves, Sec. 3.4)
     double *partials;      // observe mode: [block][kNumSums]
-    double *obs_sums;      // observe mode, FP32 arithmetic: the final sums,
-    unsigned *obs_done;    // blocks done (0 between passes)
-    int obs_solid;         // and blocks that take the solid rows
+    int obs_solid;         // observe mode, FP32 arithmetic: blocks that take the solid rows
     int residual_valid;
     T *field;              // field / init mode: per species [4][n_rows][nxp]
     // reduced-precision storage only (null otherwise)
@@ -265,7 +263,7 @@ cudaError_t launch(int Q, int storage, const void *args, int mode, int nblocks, 
 // Reference refresh from args.acc into the tables enc[s], dec[s].
 cudaError_t launch_ref(int Q, int storage, const void *args, float *const enc[3],
                        float *const dec[3], cudaStream_t s);
-// Final sums of the FP64 observation pass (with FP32 arithmetic the pass writes them itself).
+// Final sums of an observation pass from its blocks' partial sums.
 cudaError_t launch_finalize(const double *partials, int nblocks, double *sums, cudaStream_t s);
 // One more period completed by a batch (StepArgs::step_reps).
 cudaError_t launch_count_period(uint32_t *reps, cudaStream_t s);

@@ -44,6 +44,7 @@ constexpr int kFinalizeThreads = 256;
 __global__ void __launch_bounds__(kFinalizeThreads) k_finalize(const double *__restrict__ partials, int nblocks,
                                                                double *__restrict__ sums)
 {
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // the pass's partial sums
     __shared__ double red[kFinalizeThreads];
     const int k = blockIdx.x;
     const bool is_max = k == kSumResidual;
@@ -79,8 +80,16 @@ cudaError_t launch_count_period(uint32_t *reps, cudaStream_t s)
 
 cudaError_t launch_finalize(const double *partials, int nblocks, double *sums, cudaStream_t s)
 {
-    k_finalize<<<kNumSums, kFinalizeThreads, 0, s>>>(partials, nblocks, sums);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kNumSums);
+    cfg.blockDim = dim3(kFinalizeThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_finalize, partials, nblocks, sums);
 }
 
 }  // namespace klb

@@ -841,14 +841,17 @@ __device__ __forceinline__ void step_body2(const StepArgs<float> &p, int b)
 // work), so that each thread keeps its sums in registers and the FP64
 // reductions over threads run once per block instead of once per row chunk;
 // the residual's FP64 difference is formed only for cells that can raise the
-// maximum.  The last block to finish sums the blocks' partials in block
-// order (the same order every time).  Counts and distance moments of the
-// slip fit are properties of the geometry and computed on the host.
+// maximum.  k_finalize adds the blocks' partials (the same order every time).
+// Counts and distance moments of the slip fit are properties of the geometry
+// and computed on the host.
 // klb_observables, GB300, before (a block per row chunk, FP64 sums and a
 // reduction kernel over them) -> now: 512x128x128 FP32 388 -> 192 us, FP16
 // 463 -> 189; 768x192x192 FP32 1214 -> 535, FP16 1460 -> 511; 128x64x64 FP32
 // 55 -> 45; pipe R8 nx 8 43 -> 31.  L2 requests for the next item, as in the
 // step, were slower (239 us): two states stream through L2 here.
+// The final sums in a kernel of their own, launched while the pass drains,
+// instead of by the pass's last block: 512x128x128 FP32 196 -> 193 us, FP16
+// 204 -> 197, 128x64x64 52 -> 45, pipe R8 nx 8 33 -> 33.
 __device__ __forceinline__ bool finite2(const Cell2 &c, int e)
 {
     const float v[4] = {e ? c.drho.y : c.drho.x, e ? c.u[0].y : c.u[0].x, e ? c.u[1].y : c.u[1].x,
@@ -881,12 +884,6 @@ __device__ __forceinline__ int clipped2(float2 top, bool both)
     const float m = Storage<S>::kMax;
     return (top.x == m ? 1 : 0) + (both && top.y == m ? 1 : 0);
 }
-
-// Values of a block's partial row: six sums (water: u_x, momentum, mass, u_x
-// and u_x d^2 of the fit rows, u_x of the wall rows; solid: u_x, momentum,
-// mass of electrons and phonons in turn), residual, non-finite and clipped
-// species-cells.
-constexpr int kObsValues = 9;
 
 template <int Q, typename S>
 __global__ void __launch_bounds__(kBlockX, 4) k_observe2(const StepArgs<float> p)
@@ -1027,80 +1024,30 @@ __global__ void __launch_bounds__(kBlockX, 4) k_observe2(const StepArgs<float> p
     }
 
     // the block's partial row
-    __shared__ double red[kBlockX / 32][kObsValues];
-    __shared__ bool last;
+    __shared__ double red[kBlockX / 32][kNumSums];
+    if (lane < kNumSums) red[warp][lane] = 0.0;
+    __syncwarp();
     nonfinite = __reduce_add_sync(0xffffffffu, nonfinite);
     clipped = __reduce_add_sync(0xffffffffu, clipped);
     const double rm = warp_max(res.m);
+    constexpr int kW[6] = {kSumUxFluid, kSumMomW, kSumMassW, kSumFitU, kSumFitUD2, kSumWallU};
+    constexpr int kS[6] = {kSumUxE, kSumMomE, kSumMassE, kSumUxP, kSumMomP, kSumMassP};
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
         const double v = warp_sum(s[k]);
-        if (lane == 0) red[warp][k] = v;
+        if (lane == 0) red[warp][water ? kW[k] : kS[k]] = v;
     }
     if (lane == 0) {
-        red[warp][6] = rm;
-        red[warp][7] = (double)nonfinite;
-        red[warp][8] = (double)clipped;
+        red[warp][kSumResidual] = rm;
+        red[warp][kSumNonfinite] = (double)nonfinite;
+        red[warp][kSumClipped] = (double)clipped;
     }
     __syncthreads();
-    if (threadIdx.x < kObsValues) {
+    if (threadIdx.x < kNumSums) {
         const int k = threadIdx.x;
         double v = red[0][k];
-        for (int w = 1; w < wpb; ++w) v = k == 6 ? fmax(v, red[w][k]) : v + red[w][k];
+        for (int w = 1; w < wpb; ++w) v = k == kSumResidual ? fmax(v, red[w][k]) : v + red[w][k];
         p.partials[(size_t)blockIdx.x * kNumSums + k] = v;
-        __threadfence();
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(p.obs_done, 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (!last) return;
-    // the last block: warp 0 the solid blocks, the next (or the same) the water blocks
-    __threadfence();
-    if (threadIdx.x < kNumSums) p.obs_sums[threadIdx.x] = 0.0;
-    __syncthreads();
-    double *shared_res = &red[0][0];
-    for (int c = warp; c < 2; c += wpb) {
-        const int b0 = c == 0 ? 0 : p.obs_solid, b1 = c == 0 ? p.obs_solid : (int)gridDim.x;
-        double t[kObsValues];
-#pragma unroll
-        for (int k = 0; k < kObsValues; ++k) t[k] = 0.0;
-#pragma unroll 4
-        for (int b = b0 + lane; b < b1; b += 32) {
-            const double *q = p.partials + (size_t)b * kNumSums;
-#pragma unroll
-            for (int k = 0; k < kObsValues; ++k) {
-                const double v = __ldcg(q + k);
-                t[k] = k == 6 ? fmax(t[k], v) : t[k] + v;
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < kObsValues; ++k) t[k] = k == 6 ? warp_max(t[k]) : warp_sum(t[k]);
-        if (lane == 0) {
-            double *o = p.obs_sums;
-            if (c == 0) {
-                o[kSumUxE] = t[0];
-                o[kSumMomE] = t[1];
-                o[kSumMassE] = t[2];
-                o[kSumUxP] = t[3];
-                o[kSumMomP] = t[4];
-                o[kSumMassP] = t[5];
-            } else {
-                o[kSumUxFluid] = t[0];
-                o[kSumMomW] = t[1];
-                o[kSumMassW] = t[2];
-                o[kSumFitU] = t[3];
-                o[kSumFitUD2] = t[4];
-                o[kSumWallU] = t[5];
-            }
-            for (int k = 0; k < 3; ++k) shared_res[c * 3 + k] = t[6 + k];
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        p.obs_sums[kSumResidual] = fmax(shared_res[0], shared_res[3]);
-        p.obs_sums[kSumNonfinite] = shared_res[1] + shared_res[4];
-        p.obs_sums[kSumClipped] = shared_res[2] + shared_res[5];
-        *p.obs_done = 0u;  // for the next observation (stream order)
     }
 }
 
