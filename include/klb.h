@@ -344,8 +344,9 @@ klb_status klb_set_state(klb_lattice *lat, const double *g, const double *U1,
  * replayed.  The batch enqueues
  * its work on a stream of its own, ordered after and before the members'
  * stream with events.  Members stay usable on their own between batch calls
- * (observables, fields, state); stepping a member alone takes it out of phase
- * and the next batch call fails with KLB_ESTATE.
+ * (observables, fields, state, couplings): the next batch step goes on from a
+ * state or couplings replaced in between.  Stepping a member alone takes it
+ * out of phase and the next batch call fails with KLB_ESTATE.
  */
 typedef struct klb_batch klb_batch;
 

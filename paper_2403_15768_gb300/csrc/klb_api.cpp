@@ -1046,6 +1046,8 @@ struct klb_batch {
     std::vector<char> acc;        // per phase: some member accumulates x-sums
     std::vector<int64_t> base_step;  // members' steps at phase 0
     std::vector<HostState> base_state;  // members' time levels at phase 0
+    std::vector<HostState> now_state;   // and after the batch's last step
+    std::vector<klb_couplings> cp;      // members' couplings in the tables
     int64_t phase = 0;               // steps taken since phase 0
     cudaGraphExec_t graph = nullptr;
     std::string err;
@@ -1143,9 +1145,12 @@ klb_status build_tables(klb_batch *B, int width)
     B->phase = 0;
     B->base_step.resize(n);
     B->base_state.resize(n);
+    B->now_state.resize(n);
+    B->cp.resize(n);
     for (int m = 0; m < n; ++m) {
         B->base_step[m] = B->mem[m]->st.step;
-        B->base_state[m] = B->mem[m]->st;
+        B->base_state[m] = B->now_state[m] = B->mem[m]->st;
+        B->cp[m] = B->mem[m]->cp;
     }
     destroy_graph(B);
     return KLB_OK;
@@ -1203,6 +1208,13 @@ bool in_phase(const klb_batch *B)
     return true;
 }
 
+// Whether two time levels at the same step read and write the same buffers.
+bool same_level(const HostState &a, const HostState &b)
+{
+    return a.cur == b.cur && a.gen_buf[0] == b.gen_buf[0] && a.gen_buf[1] == b.gen_buf[1] &&
+           a.refresh_pending == b.refresh_pending;
+}
+
 // Whether every member stands where the tables' phase 0 assumed.  The step
 // pattern repeats after a period from any time level but one: right after
 // an initialisation of 16-bit storage no reference refresh is pending at a
@@ -1210,13 +1222,34 @@ bool in_phase(const klb_batch *B)
 // period.
 bool tables_repeat(const klb_batch *B)
 {
+    for (size_t m = 0; m < B->mem.size(); ++m)
+        if (!same_level(B->mem[m]->st, B->base_state[m])) return false;
+    return true;
+}
+
+// Whether the members are as the batch left them: klb_set_state at the same
+// step resets a member's buffer and reference generation, and couplings are
+// part of the argument records.
+bool untouched(const klb_batch *B)
+{
     for (size_t m = 0; m < B->mem.size(); ++m) {
-        const HostState &a = B->mem[m]->st, &b = B->base_state[m];
-        if (a.cur != b.cur || a.gen_buf[0] != b.gen_buf[0] || a.gen_buf[1] != b.gen_buf[1] ||
-            a.refresh_pending != b.refresh_pending)
+        const klb_couplings &a = B->mem[m]->cp, &b = B->cp[m];
+        if (!same_level(B->mem[m]->st, B->now_state[m]) || a.g_we != b.g_we || a.g_wp != b.g_wp ||
+            a.g_ep != b.g_ep || a.g_ec != b.g_ec || a.g_pc != b.g_pc)
             return false;
     }
     return true;
+}
+
+// Advances the members' time levels by steps that the batch has enqueued.
+void advance_members(klb_batch *B, int steps)
+{
+    for (size_t m = 0; m < B->mem.size(); ++m) {
+        HostState &h = B->mem[m]->st;
+        for (int j = 0; j < steps; ++j) advance(h, plan_step(h, reduced(B->mem[m])));
+        B->now_state[m] = h;
+    }
+    B->phase += steps;
 }
 
 // Runs nsteps phases on the batch stream, replaying the graph for whole
@@ -1237,17 +1270,12 @@ klb_status run_steps(klb_batch *B, int64_t nsteps, bool use_graph)
                 if (st != KLB_OK) return st;
             }
             KLB_BCUDA(B, cudaGraphLaunch(B->graph, B->stream));
-            for (klb_lattice *L : B->mem) {
-                HostState &h = L->st;
-                for (int j = 0; j < B->period; ++j) advance(h, plan_step(h, reduced(L)));
-            }
-            B->phase += B->period;
+            advance_members(B, B->period);
             nsteps -= B->period;
             continue;
         }
         KLB_BCUDA(B, launch_phase(B, k));
-        for (klb_lattice *L : B->mem) advance(L->st, plan_step(L->st, reduced(L)));
-        ++B->phase;
+        advance_members(B, 1);
         --nsteps;
     }
     return KLB_OK;
@@ -1344,6 +1372,10 @@ klb_status klb_batch_step(klb_batch *B, int64_t nsteps)
     if (nsteps < 0) return bfail(B, KLB_EINVAL, "nsteps must be >= 0");
     if (!in_phase(B))
         return bfail(B, KLB_ESTATE, "a member was stepped outside the batch; form the batch again");
+    if (nsteps > 0 && !untouched(B)) {
+        const klb_status st = build_tables(B, B->width);
+        if (st != KLB_OK) return st;
+    }
     KLB_BCUDA(B, cudaEventRecord(B->ev_in, B->user));
     KLB_BCUDA(B, cudaStreamWaitEvent(B->stream, B->ev_in, 0));
     klb_status st = run_steps(B, nsteps, true);
