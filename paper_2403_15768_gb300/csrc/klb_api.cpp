@@ -89,27 +89,45 @@ size_t state_bytes(const klb_lattice *L)
     return 2 * (L->plan.pop_bytes[0] + L->plan.pop_bytes[1] + L->plan.pop_bytes[2]);
 }
 
-// Kernel arguments for the time level `st` (the step about to run, or the
-// one observed); the step kernel runs blocks of sbx threads and touches
-// all_bytes of state buffers per launch.
+// Kernel arguments that follow the time level `st` (the step about to run, or
+// the one observed).
 template <typename T>
-void fill_args_at(const klb_lattice *L, const HostState &st, int sbx, bool ep, size_t all_bytes, StepArgs<T> &a)
+void fill_level(const klb_lattice *L, const HostState &st, StepArgs<T> &a)
 {
-    const Geometry &g = L->geo;
     const MemoryPlan &p = L->plan;
-    std::memset(&a, 0, sizeof a);
     const int64_t n = st.step;
     for (int s = 0; s < 3; ++s) {
         a.in[s] = dev(L, p.pop[st.cur][s]);
         a.out[s] = dev(L, p.pop[1 - st.cur][s]);
         a.in_prev[s] = dev(L, p.pop[1 - st.cur][s]);
     }
-    if (reduced(L)) {
+    if (reduced(L))
         for (int s = 0; s < 3; ++s) {
             a.dec_in[s] = (const float *)dev(L, p.ref_dec[st.gen_buf[st.cur]][s]);
             a.dec_prev[s] = (const float *)dev(L, p.ref_dec[st.gen_buf[1 - st.cur]][s]);
             a.enc_out[s] = (const float *)dev(L, p.ref_enc[st.gen_buf[st.cur]][s]);
         }
+    for (int c = 0; c < 2; ++c) {
+        a.U0[c] = (T *)dev(L, p.U[slot_of(n)][c]);
+        a.U1[c] = (const T *)dev(L, p.U[slot_of(n - 1)][c]);
+        a.U2[c] = (const T *)dev(L, p.U[slot_of(n - 2)][c]);
+        a.U3[c] = (const T *)dev(L, p.U[slot_of(n - 3)][c]);
+    }
+    a.residual_valid = st.since_reset >= 2;
+    a.step_lo = (uint32_t)((uint64_t)n & 0xffffffffu);
+    a.step_hi = (uint32_t)((uint64_t)n >> 32);
+}
+
+// All kernel arguments for the time level `st`; the step kernel runs blocks
+// of sbx threads and touches all_bytes of state buffers per launch.
+template <typename T>
+void fill_args_at(const klb_lattice *L, const HostState &st, int sbx, bool ep, size_t all_bytes, StepArgs<T> &a)
+{
+    const Geometry &g = L->geo;
+    const MemoryPlan &p = L->plan;
+    std::memset((void *)&a, 0, sizeof a);
+    fill_level(L, st, a);
+    if (reduced(L)) {
         a.scale = L->desc.storage == KLB_FP16_DEV ? kFp16Scale : 1.0f;
         a.inv_scale = 1.0f / a.scale;
         a.acc = (float *)dev(L, p.acc);
@@ -118,10 +136,6 @@ void fill_args_at(const klb_lattice *L, const HostState &st, int sbx, bool ep, s
     }
     for (int c = 0; c < 2; ++c) {
         a.rows[c] = (const RowInfo *)dev(L, p.rows[c]);
-        a.U0[c] = (T *)dev(L, p.U[slot_of(n)][c]);
-        a.U1[c] = (const T *)dev(L, p.U[slot_of(n - 1)][c]);
-        a.U2[c] = (const T *)dev(L, p.U[slot_of(n - 2)][c]);
-        a.U3[c] = (const T *)dev(L, p.U[slot_of(n - 3)][c]);
         a.n_rows[c] = (int)g.rows[c].size();
         a.n_slots[c] = (int)g.slot_row[c].size();
     }
@@ -157,14 +171,11 @@ void fill_args_at(const klb_lattice *L, const HostState &st, int sbx, bool ep, s
     a.g_pc = (T)L->cp.g_pc;
     a.q_p = (T)(d.phonon_eq == KLB_PHONON_WAVE ? 0.0 : 1.0);
     a.partials = (double *)dev(L, p.partials);
-    a.residual_valid = st.since_reset >= 2;
     a.field = (T *)dev(L, p.field);
     const double om = 1.0 / d.tau_w;
     a.noise_amp = (T)(L->kT > 0.0 ? std::sqrt(3.0 * d.rho0 * L->kT * om * (2.0 - om)) : 0.0);
     a.key[0] = (uint32_t)(L->seed & 0xffffffffu);
     a.key[1] = (uint32_t)(L->seed >> 32);
-    a.step_lo = (uint32_t)((uint64_t)n & 0xffffffffu);
-    a.step_hi = (uint32_t)((uint64_t)n >> 32);
     a.bounds_err = (unsigned *)dev(L, p.bounds);
     for (int s = 0; s < 3; ++s) a.ck[s] = collide_k(g.Q, (float)a.om[s]);
     a.ahead = step_ahead(g.Q, d.storage, g.nxp, all_bytes);
@@ -1039,9 +1050,10 @@ struct klb_batch {
     int width = kBlockX;
     int nblocks = 0;
     bool ep = false;
-    size_t args_size = 0, table_off = 0, prefix_off = 0, reps_off = 0;
-    std::vector<char> table;      // host copies of the argument tables and the block prefix
+    size_t rec_size = 0, table_off = 0, prefix_off = 0, reps_off = 0;
+    std::vector<char> table;      // argument records [phase][member], the block prefix
     std::vector<int> prefix;
+    std::vector<CollideK> ck;     // and the collision constants, three per member
     std::vector<StepPlan> plans;  // per (phase, member)
     std::vector<char> acc;        // per phase: some member accumulates x-sums
     std::vector<int64_t> base_step;  // members' steps at phase 0
@@ -1069,16 +1081,19 @@ klb_status bfail(klb_batch *B, klb_status st, const std::string &msg)
 
 int batch_period(int storage) { return reduced_storage(storage) ? 6 * 2 * kRefEvery : 6; }
 
-size_t args_size(int storage) { return storage == KLB_FP64 ? sizeof(StepArgs<double>) : sizeof(StepArgs<float>); }
+size_t rec_size(int storage) { return storage == KLB_FP64 ? sizeof(StepRecord<double>) : sizeof(StepRecord<float>); }
 
-// Batch buffer: argument tables [phase][member], block prefix, period count.
+// Batch buffer: period count, and for batches that may be launched over
+// device copies (batch_by_table) the argument records [phase][member] and
+// the block prefix.
 size_t batch_layout(int n, int storage, size_t *table_off, size_t *prefix_off, size_t *reps_off)
 {
-    const size_t tb = (size_t)batch_period(storage) * n * args_size(storage);
-    *table_off = 0;
-    *prefix_off = (tb + 255) / 256 * 256;
-    *reps_off = *prefix_off + ((size_t)(n + 1) * sizeof(int) + 255) / 256 * 256;
-    return *reps_off + 256;
+    *reps_off = 0;
+    *prefix_off = 256;
+    *table_off = 256;
+    if (n <= kBatchParams) return 256;
+    *table_off += ((size_t)(n + 1) * sizeof(int) + 255) / 256 * 256;
+    return *table_off + ((size_t)batch_period(storage) * n * rec_size(storage) + 255) / 256 * 256;
 }
 
 void destroy_graph(klb_batch *B)
@@ -1087,58 +1102,62 @@ void destroy_graph(klb_batch *B)
     B->graph = nullptr;
 }
 
-// Per-phase argument tables for block width `width`, from each member's own
-// time level now (phase 0), the block prefix, and the phase plans.  Every
-// member's step pattern repeats after the batch period whatever its step
-// count, so members may stand at different time levels.  A launch
-// accumulates reference x-sums when any member needs them; the x-sums are
-// stored, not added, so an extra pass leaves the other members' refreshes
-// unchanged.
+// A member's argument records of every phase, from its time level now: the
+// arguments once, then what follows the time level.
+template <typename T>
+void fill_records(klb_batch *B, int m, int width, size_t all_bytes)
+{
+    const klb_lattice *L = B->mem[m];
+    const int n = (int)B->mem.size(), P = B->period;
+    StepArgs<T> a;
+    fill_args_at(L, L->st, width, B->ep, all_bytes, a);
+    a.step_reps = (const uint32_t *)(B->base + B->reps_off);
+    a.step_period = P;
+    for (int s = 0; s < 3; ++s) B->ck[3 * m + s] = a.ck[s];
+    HostState st = L->st;
+    for (int k = 0; k < P; ++k) {
+        const StepPlan sp = plan_step(st, reduced(L));
+        B->plans[(size_t)k * n + m] = sp;
+        B->acc[k] |= (char)sp.acc;
+        fill_level(L, st, a);
+        set_enc(L, &a, sp.outgen);
+        reinterpret_cast<StepRecord<T> *>(B->table.data())[(size_t)k * n + m] = a;
+        advance(st, sp);
+    }
+}
+
+// Argument records for block width `width`, from each member's own time level
+// now (phase 0), the block prefix, and the phase plans.  Every member's step
+// pattern repeats after the batch period whatever its step count, so members
+// may stand at different time levels.  A launch accumulates reference x-sums
+// when any member needs them; the x-sums are stored, not added, so an extra
+// pass leaves the other members' refreshes unchanged.
 klb_status build_tables(klb_batch *B, int width)
 {
     const int n = (int)B->mem.size(), P = B->period;
-    std::vector<char> &host = B->table;
     std::vector<int> &prefix = B->prefix;
-    host.assign((size_t)P * n * B->args_size, 0);
+    B->table.resize((size_t)P * n * B->rec_size);
+    B->ck.resize(3 * (size_t)n);
     prefix.assign(n + 1, 0);
-    B->plans.assign((size_t)P * n, StepPlan{0, false, false});
+    B->plans.resize((size_t)P * n);
     B->acc.assign(P, 0);
     size_t all_bytes = 0;
     for (const klb_lattice *L : B->mem) all_bytes += state_bytes(L);
     for (int m = 0; m < n; ++m) {
-        const klb_lattice *L = B->mem[m];
-        HostState st = L->st;
-        for (int k = 0; k < P; ++k) {
-            const StepPlan sp = plan_step(st, reduced(L));
-            B->plans[(size_t)k * n + m] = sp;
-            B->acc[k] |= (char)sp.acc;
-            char *slot = host.data() + ((size_t)k * n + m) * B->args_size;
-            const uint32_t *reps = (const uint32_t *)(B->base + B->reps_off);
-            if (B->storage == KLB_FP64) {
-                StepArgs<double> a;
-                fill_args_at(L, st, width, B->ep, all_bytes, a);
-                a.step_reps = reps;
-                a.step_period = P;
-                std::memcpy(slot, &a, sizeof a);
-            } else {
-                StepArgs<float> a;
-                fill_args_at(L, st, width, B->ep, all_bytes, a);
-                a.step_reps = reps;
-                a.step_period = P;
-                if (reduced(L))
-                    for (int s = 0; s < 3; ++s) a.enc_out[s] = (const float *)dev(L, L->plan.ref_enc[sp.outgen][s]);
-                std::memcpy(slot, &a, sizeof a);
-            }
-            advance(st, sp);
-        }
-        const int sto = L->desc.storage;
-        prefix[m + 1] = prefix[m] + step_blocks(L->geo.nx, (int)L->geo.rows[kFluid].size(),
-                                                (int)L->geo.rows[kSolid].size(), width, sto, B->ep);
+        if (B->storage == KLB_FP64)
+            fill_records<double>(B, m, width, all_bytes);
+        else
+            fill_records<float>(B, m, width, all_bytes);
+        const Geometry &g = B->mem[m]->geo;
+        prefix[m + 1] = prefix[m] + step_blocks(g.nx, (int)g.rows[kFluid].size(), (int)g.rows[kSolid].size(), width,
+                                                B->storage, B->ep);
     }
     KLB_BCUDA(B, cudaStreamSynchronize(B->stream));
-    KLB_BCUDA(B, cudaMemcpy(B->base + B->table_off, host.data(), host.size(), cudaMemcpyHostToDevice));
-    KLB_BCUDA(B, cudaMemcpy(B->base + B->prefix_off, prefix.data(), prefix.size() * sizeof(int),
-                            cudaMemcpyHostToDevice));
+    if (batch_by_table(n, prefix[n])) {
+        KLB_BCUDA(B, cudaMemcpy(B->base + B->table_off, B->table.data(), B->table.size(), cudaMemcpyHostToDevice));
+        KLB_BCUDA(B, cudaMemcpy(B->base + B->prefix_off, prefix.data(), prefix.size() * sizeof(int),
+                                cudaMemcpyHostToDevice));
+    }
     KLB_BCUDA(B, cudaMemset(B->base + B->reps_off, 0, sizeof(uint32_t)));
     B->width = width;
     B->nblocks = prefix[n];
@@ -1171,9 +1190,9 @@ cudaError_t launch_phase(klb_batch *B, int k)
         L->stream = keep;
         if (e != cudaSuccess) return e;
     }
-    const size_t at = (size_t)k * n * B->args_size;
+    const size_t at = (size_t)k * n * B->rec_size;
     const BatchLaunch b{B->table.data() + at, B->base + B->table_off + at, B->prefix.data(),
-                        (const int *)(B->base + B->prefix_off), (int)n, B->width, B->acc[k] != 0, B->ep};
+                        (const int *)(B->base + B->prefix_off), B->ck.data(), (int)n, B->width, B->acc[k] != 0, B->ep};
     cudaError_t e = launch_batch(B->Q, B->storage, b, B->stream);
     if (e == cudaSuccess && k == B->period - 1) e = launch_count_period((uint32_t *)(B->base + B->reps_off), B->stream);
     return e;
@@ -1322,7 +1341,7 @@ klb_status klb_batch_create(klb_lattice *const *members, int n, void *dev_buf, s
     B->Q = members[0]->geo.Q;
     B->storage = members[0]->desc.storage;
     B->period = batch_period(B->storage);
-    B->args_size = args_size(B->storage);
+    B->rec_size = rec_size(B->storage);
     const size_t need = batch_layout(n, B->storage, &B->table_off, &B->prefix_off, &B->reps_off);
     if (!dev_buf || ((uintptr_t)dev_buf & 255u)) {
         delete B;

@@ -202,17 +202,17 @@ inline __host__ __device__ CollideK collide_k(int Q, float om)
     return c;
 }
 
-// Kernel arguments.  T is the arithmetic type (float or double); the
-// populations are stored as T, or as FP16/BF16 against per-row references.
+// What a step reads of its lattice: the record that a batch keeps per phase
+// and member.  T is the arithmetic type (float or double); the populations
+// are stored as T, or as FP16/BF16 against per-row references.
 template <typename T>
-struct alignas(16) StepArgs {
+struct alignas(16) StepRecord {
     const void *in[3];     // current state, per species
     void *out[3];          // next state (step and init modes)
-    const void *in_prev[3];  // previous state (observe mode, residual)
     const RowInfo *rows[2];
-    const T *U1[2], *U2[2], *U3[2];  // lagged velocities u(n-1), u(n-2), u(n-3)
-    T *U0[2];                        // u(n) written here (step mode)
-    int nx, nxp, nchunk, nbw;        // nchunk = x chunks of blockDim.x per row; nbw = water blocks
+    const T *U1[2], *U2[2];  // lagged velocities u(n-1), u(n-2)
+    T *U0[2];                // u(n) written here (step mode)
+    int nx, nxp;
     int snchunk, split;              // FP64 step: x chunks of blockDim.x per row; one species per solid block
     int nseg64;                      // 64-wide x segments per row
     uint32_t seg_mul, seg_shift;     // n / nseg64 = n seg_mul >> seg_shift for 0 <= n < 2^31
@@ -223,13 +223,9 @@ struct alignas(16) StepArgs {
     T rho0, om[3], G[3];
     T g_we, g_wp, g_ep, g_ec, g_pc;
     T q_p;                 // phonons: 1 second-order equilibrium, 0 linear (damped waves, Sec. 3.4)
-    double *partials;      // observe mode: [block][kNumSums]
-    int obs_solid;         // observe mode, FP32 arithmetic: blocks that take the solid rows
-    int residual_valid;
-    T *field;              // field / init mode: per species [4][n_rows][nxp]
     // reduced-precision storage only (null otherwise)
-    const float *dec_in[3], *dec_prev[3];  // references of pulled populations
-    const float *enc_out[3];               // references of stored populations
+    const float *dec_in[3];   // references of pulled populations
+    const float *enc_out[3];  // references of stored populations
     float scale, inv_scale;
     float *acc;            // x-sums of g* per 32-wide segment [segment][2Q]
     // thermal fluctuations of the water (step with noise only)
@@ -242,8 +238,22 @@ struct alignas(16) StepArgs {
     const uint32_t *step_reps;
     int step_period;
     int ahead;             // rows ahead whose populations the step asks L2 for (step_ahead; 0: none)
-    CollideK ck[3];        // FP32 arithmetic: collision constants per species
     unsigned *bounds_err;  // debug builds: first out-of-range index site
+};
+
+// Kernel arguments: the record, what is the same in every step of a lattice
+// and formed from it, and what the other passes read.
+template <typename T>
+struct alignas(16) StepArgs : StepRecord<T> {
+    CollideK ck[3];          // FP32 arithmetic: collision constants per species
+    const void *in_prev[3];  // observe mode: previous state and its references (residual),
+    const float *dec_prev[3];
+    const T *U3[2];          // u(n-3),
+    double *partials;        // [block][kNumSums],
+    int obs_solid;           // with FP32 arithmetic the blocks that take the solid rows
+    int residual_valid;
+    int nchunk, nbw;         // observe, field and init modes: x chunks of blockDim.x per row, water blocks
+    T *field;                // field / init mode: per species [4][n_rows][nxp]
 };
 
 enum Mode {
@@ -267,19 +277,21 @@ cudaError_t launch_ref(int Q, int storage, const void *args, float *const enc[3]
 cudaError_t launch_finalize(const double *partials, int nblocks, double *sums, cudaStream_t s);
 // One more period completed by a batch (StepArgs::step_reps).
 cudaError_t launch_count_period(uint32_t *reps, cudaStream_t s);
-// One step of many lattices: argument records (host and device copies) and
-// first block of each lattice (prefix[n] = total blocks).  Up to
-// kBatchParams records go as kernel parameters (32 KB in all); more
+// One step of many lattices: argument records and first block of each lattice
+// (prefix[n] = total blocks), and the collision constants, three per lattice.
+// Up to kBatchParams records go as kernel parameters (32 KB in all); more
 // lattices take several such launches if the step has at least kGroupBlocks
-// blocks, else one launch over the device table: a launch waits for the one
-// before it.  One launch over the table -> several: 64 channels of a sweep
-// FP32 2410 -> 2310 us, FP16 2305 -> 2162; 100 pipes of R 6-9, nx 8 (8800
-// blocks) FP32 84.7 -> 82.8, FP16 127.2 -> 125.9.
+// blocks, else one launch over the device copies (batch_by_table): a launch
+// waits for the one before it.  One launch over the table -> several: 64
+// channels of a sweep FP32 2410 -> 2310 us, FP16 2305 -> 2162; 100 pipes of
+// R 6-9, nx 8 (8800 blocks) FP32 84.7 -> 82.8, FP16 127.2 -> 125.9.
 constexpr int kBatchParams = 36;
 constexpr int kGroupBlocks = 4000;
+inline bool batch_by_table(int n, int blocks) { return n > kBatchParams && blocks < kGroupBlocks; }
 struct BatchLaunch {
     const void *table, *dev_table;
     const int *prefix, *dev_prefix;
+    const CollideK *ck;
     int n, width;
     bool acc, ep;
 };

@@ -1092,17 +1092,20 @@ cudaError_t launch_step(void (*kernel)(A), int nblocks, int bx, cudaStream_t s, 
 // arguments.
 template <int Q, typename T, typename S, bool ACC, bool EP>
 __global__ void __launch_bounds__(kBlockX, (step_min_blocks<T, S, EP>()))
-    k_step_batch(const StepArgs<T> *__restrict__ table, const int *__restrict__ prefix, int n)
+    k_step_batch(const StepRecord<T> *__restrict__ table, const int *__restrict__ prefix, int n)
 {
     pdl_launch_dependents();
     __shared__ StepArgs<T> sp;
     int c = 0;
     for (int m = 1 + ((int)threadIdx.x & 31); m < n; m += 32) c += __ldg(prefix + m) <= (int)blockIdx.x;
     const int lid = (int)__reduce_add_sync(0xffffffffu, (unsigned)c);
-    static_assert(sizeof(StepArgs<T>) % 16 == 0, "argument record in 16-byte words");
+    static_assert(sizeof(StepRecord<T>) % 16 == 0, "argument record in 16-byte words");
     const int4 *src = reinterpret_cast<const int4 *>(table + lid);
-    int4 *dst = reinterpret_cast<int4 *>(&sp);
-    for (int k = threadIdx.x; k < (int)(sizeof(StepArgs<T>) / 16); k += blockDim.x) dst[k] = __ldg(src + k);
+    int4 *dst = reinterpret_cast<int4 *>(static_cast<StepRecord<T> *>(&sp));
+    for (int k = threadIdx.x; k < (int)(sizeof(StepRecord<T>) / 16); k += blockDim.x) dst[k] = __ldg(src + k);
+    if constexpr (sizeof(T) == 4) {
+        if (threadIdx.x < 3) sp.ck[threadIdx.x] = collide_k(Q, __ldg(&table[lid].om[threadIdx.x]));
+    }
     __syncthreads();
     step_cells_body<Q, T, S, ACC, false, EP>(sp, (int)blockIdx.x - __ldg(prefix + lid));
 }
@@ -1257,17 +1260,20 @@ cudaError_t launch_batch_form(const BatchLaunch &b, cudaStream_t s)
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     const int total = b.prefix[b.n];
-    const int groups = (b.n + kBatchParams - 1) / kBatchParams;
-    if (groups > 1 && total < kGroupBlocks) {
+    if (batch_by_table(b.n, total)) {
         cfg.gridDim = dim3((unsigned)total);
-        return cudaLaunchKernelEx(&cfg, k_step_batch<Q, T, S, ACC, EP>, static_cast<const StepArgs<T> *>(b.dev_table),
+        return cudaLaunchKernelEx(&cfg, k_step_batch<Q, T, S, ACC, EP>, static_cast<const StepRecord<T> *>(b.dev_table),
                                   b.dev_prefix, b.n);
     }
+    const int groups = (b.n + kBatchParams - 1) / kBatchParams;
     for (int g = 0; g < groups; ++g) {
         const int m0 = (int)((long long)b.n * g / groups), m1 = (int)((long long)b.n * (g + 1) / groups);
         BatchTable<T> tb;
         tb.n = m1 - m0;
-        std::memcpy(tb.a, static_cast<const StepArgs<T> *>(b.table) + m0, tb.n * sizeof(StepArgs<T>));
+        for (int m = m0; m < m1; ++m) {
+            static_cast<StepRecord<T> &>(tb.a[m - m0]) = static_cast<const StepRecord<T> *>(b.table)[m];
+            for (int s = 0; s < 3; ++s) tb.a[m - m0].ck[s] = b.ck[3 * m + s];
+        }
         for (int m = m0; m <= m1; ++m) tb.prefix[m - m0] = b.prefix[m] - b.prefix[m0];
         cfg.gridDim = dim3((unsigned)tb.prefix[tb.n]);
         const cudaError_t e = cudaLaunchKernelEx(&cfg, k_step_group<Q, T, S, ACC, EP>, tb);
