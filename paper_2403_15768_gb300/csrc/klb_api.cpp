@@ -1049,7 +1049,7 @@ struct klb_batch {
     int period = 6;
     int width = kBlockX;
     int nblocks = 0;
-    bool ep = false;
+    bool ep = false, by_table = false;
     size_t rec_size = 0, table_off = 0, prefix_off = 0, reps_off = 0;
     std::vector<char> table;      // argument records [phase][member], the block prefix
     std::vector<int> prefix;
@@ -1153,7 +1153,7 @@ klb_status build_tables(klb_batch *B, int width)
                                                 B->storage, B->ep);
     }
     KLB_BCUDA(B, cudaStreamSynchronize(B->stream));
-    if (batch_by_table(n, prefix[n])) {
+    if (B->by_table) {
         KLB_BCUDA(B, cudaMemcpy(B->base + B->table_off, B->table.data(), B->table.size(), cudaMemcpyHostToDevice));
         KLB_BCUDA(B, cudaMemcpy(B->base + B->prefix_off, prefix.data(), prefix.size() * sizeof(int),
                                 cudaMemcpyHostToDevice));
@@ -1192,7 +1192,7 @@ cudaError_t launch_phase(klb_batch *B, int k)
     }
     const size_t at = (size_t)k * n * B->rec_size;
     const BatchLaunch b{B->table.data() + at, B->base + B->table_off + at, B->prefix.data(),
-                        (const int *)(B->base + B->prefix_off), B->ck.data(), (int)n, B->width, B->acc[k] != 0, B->ep};
+                        (const int *)(B->base + B->prefix_off), B->ck.data(), (int)n, B->width, B->acc[k] != 0, B->ep, B->by_table};
     cudaError_t e = launch_batch(B->Q, B->storage, b, B->stream);
     if (e == cudaSuccess && k == B->period - 1) e = launch_count_period((uint32_t *)(B->base + B->reps_off), B->stream);
     return e;
@@ -1364,17 +1364,18 @@ klb_status klb_batch_create(klb_lattice *const *members, int n, void *dev_buf, s
         return fail(nullptr, KLB_ECUDA, m);
     }
     int w = kBlockX;
+    long long items[2] = {0, 0};
+    for (klb_lattice *L : B->mem) {
+        const Geometry &g = L->geo;
+        for (int e = 0; e < 2; ++e) items[e] += step_items(g.nx, g.rows[kFluid].size(), g.rows[kSolid].size(), e != 0);
+    }
     if (B->storage == KLB_FP64) {
         for (klb_lattice *L : B->mem) w = std::min(w, L->plan.sbx);
     } else {
-        long long items[2] = {0, 0};
-        for (klb_lattice *L : B->mem) {
-            const Geometry &g = L->geo;
-            for (int e = 0; e < 2; ++e) items[e] += step_items(g.nx, g.rows[kFluid].size(), g.rows[kSolid].size(), e != 0);
-        }
         B->ep = step_ep(items[1]);
         w = step_width(items[B->ep]);
     }
+    B->by_table = batch_by_table(n, B->storage, items[B->ep]);
     klb_status st = build_tables(B, w);
     if (st != KLB_OK) {
         std::string m = B->err;

@@ -279,21 +279,31 @@ cudaError_t launch_finalize(const double *partials, int nblocks, double *sums, c
 cudaError_t launch_count_period(uint32_t *reps, cudaStream_t s);
 // One step of many lattices: argument records and first block of each lattice
 // (prefix[n] = total blocks), and the collision constants, three per lattice.
-// Up to kBatchParams records go as kernel parameters (32 KB in all); more
-// lattices take several such launches if the step has at least kGroupBlocks
-// blocks, else one launch over the device copies (batch_by_table): a launch
-// waits for the one before it.  One launch over the table -> several: 64
-// channels of a sweep FP32 2410 -> 2310 us, FP16 2305 -> 2162; 100 pipes of
-// R 6-9, nx 8 (8800 blocks) FP32 84.7 -> 82.8, FP16 127.2 -> 125.9.
+// Up to kBatchParams records go as kernel parameters (32 KB in all).  More
+// lattices take several such launches, or one over device copies of the
+// records (batch_by_table).  A launch waits for the one before it, so several
+// pay only when each fills the chip (20 warps on each of 152 SMs) some times
+// over: kGroupItems items (warps) in each.  One launch -> several, us per
+// step, GB300, FP32 / FP16, by items per launch: 1333 (400 D2Q9 slabs 64x40)
+// 24.7 -> 57.0 / 72.2 -> 104; 4466 (400 pipes R 4-5, nx 3) 145 -> 165 / 229 ->
+// 245; 4824 (72 of them) 25.9 -> 26.1 / 36.2 -> 39.0; 7020 (40 pipes R 6-9, nx
+// 8) 35.6 -> 35.3 / 42.4 -> 42.9; 9065 (40 sweep channels at a quarter) 44.1 ->
+// 43.0 / 49.2 -> 49.3; 11700 (100 pipes R 6-9) 87.9 -> 83.0 / 117 -> 113;
+// 61200 (40 channels at half) 232 -> 214 / 238 -> 219.  FP64, which the FP64
+// pipe bounds, takes one launch throughout (61200: 427 -> 450 at a quarter).
 constexpr int kBatchParams = 36;
-constexpr int kGroupBlocks = 4000;
-inline bool batch_by_table(int n, int blocks) { return n > kBatchParams && blocks < kGroupBlocks; }
+constexpr long long kGroupItems = 8000;
+inline int batch_groups(int n) { return (n + kBatchParams - 1) / kBatchParams; }
+inline bool batch_by_table(int n, int storage, long long items)
+{
+    return n > kBatchParams && (storage == KLB_FP64 || items < kGroupItems * batch_groups(n));
+}
 struct BatchLaunch {
     const void *table, *dev_table;
     const int *prefix, *dev_prefix;
     const CollideK *ck;
     int n, width;
-    bool acc, ep;
+    bool acc, ep, by_table;
 };
 cudaError_t launch_batch(int Q, int storage, const BatchLaunch &b, cudaStream_t s);
 

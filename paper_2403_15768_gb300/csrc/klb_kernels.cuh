@@ -1259,13 +1259,12 @@ cudaError_t launch_batch_form(const BatchLaunch &b, cudaStream_t s)
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const int total = b.prefix[b.n];
-    if (batch_by_table(b.n, total)) {
-        cfg.gridDim = dim3((unsigned)total);
+    if (b.by_table) {
+        cfg.gridDim = dim3((unsigned)b.prefix[b.n]);
         return cudaLaunchKernelEx(&cfg, k_step_batch<Q, T, S, ACC, EP>, static_cast<const StepRecord<T> *>(b.dev_table),
                                   b.dev_prefix, b.n);
     }
-    const int groups = (b.n + kBatchParams - 1) / kBatchParams;
+    const int groups = batch_groups(b.n);
     for (int g = 0; g < groups; ++g) {
         const int m0 = (int)((long long)b.n * g / groups), m1 = (int)((long long)b.n * (g + 1) / groups);
         BatchTable<T> tb;
