@@ -177,7 +177,7 @@ void fill_args_at(const klb_lattice *L, const HostState &st, int sbx, bool ep, s
     a.key[0] = (uint32_t)(L->seed & 0xffffffffu);
     a.key[1] = (uint32_t)(L->seed >> 32);
     a.bounds_err = (unsigned *)dev(L, p.bounds);
-    for (int s = 0; s < 3; ++s) a.ck[s] = collide_k(g.Q, (float)a.om[s]);
+    for (int s = 0; s < 3; ++s) a.ck.s[s] = collide_k(g.Q, (float)a.om[s]);
     a.ahead = step_ahead(g.Q, d.storage, g.nxp, all_bytes);
 }
 
@@ -1050,10 +1050,10 @@ struct klb_batch {
     int width = kBlockX;
     int nblocks = 0;
     bool ep = false, by_table = false;
-    size_t rec_size = 0, table_off = 0, prefix_off = 0, reps_off = 0;
+    size_t rec_size = 0, table_off = 0, prefix_off = 0, ck_off = 0, reps_off = 0;
     std::vector<char> table;      // argument records [phase][member], the block prefix
     std::vector<int> prefix;
-    std::vector<CollideK> ck;     // and the collision constants, three per member
+    std::vector<CollideSet> ck;   // and the members' collision constants
     std::vector<StepPlan> plans;  // per (phase, member)
     std::vector<char> acc;        // per phase: some member accumulates x-sums
     std::vector<int64_t> base_step;  // members' steps at phase 0
@@ -1084,16 +1084,17 @@ int batch_period(int storage) { return reduced_storage(storage) ? 6 * 2 * kRefEv
 size_t rec_size(int storage) { return storage == KLB_FP64 ? sizeof(StepRecord<double>) : sizeof(StepRecord<float>); }
 
 // Batch buffer: period count, and for batches that may be launched over
-// device copies (batch_by_table) the argument records [phase][member] and
-// the block prefix.
-size_t batch_layout(int n, int storage, size_t *table_off, size_t *prefix_off, size_t *reps_off)
+// device copies (batch_by_table) the block prefix, the collision constants
+// (FP32 arithmetic) and the argument records [phase][member].
+size_t batch_layout(int n, int storage, size_t *table_off, size_t *prefix_off, size_t *ck_off, size_t *reps_off)
 {
+    auto round_up = [](size_t b) { return (b + 255) / 256 * 256; };
     *reps_off = 0;
-    *prefix_off = 256;
-    *table_off = 256;
+    *prefix_off = *ck_off = *table_off = 256;
     if (n <= kBatchParams) return 256;
-    *table_off += ((size_t)(n + 1) * sizeof(int) + 255) / 256 * 256;
-    return *table_off + ((size_t)batch_period(storage) * n * rec_size(storage) + 255) / 256 * 256;
+    *ck_off = *prefix_off + round_up((size_t)(n + 1) * sizeof(int));
+    *table_off = *ck_off + (storage == KLB_FP64 ? 0 : round_up((size_t)n * sizeof(CollideSet)));
+    return *table_off + round_up((size_t)batch_period(storage) * n * rec_size(storage));
 }
 
 void destroy_graph(klb_batch *B)
@@ -1113,7 +1114,7 @@ void fill_records(klb_batch *B, int m, int width, size_t all_bytes)
     fill_args_at(L, L->st, width, B->ep, all_bytes, a);
     a.step_reps = (const uint32_t *)(B->base + B->reps_off);
     a.step_period = P;
-    for (int s = 0; s < 3; ++s) B->ck[3 * m + s] = a.ck[s];
+    B->ck[m] = a.ck;
     HostState st = L->st;
     for (int k = 0; k < P; ++k) {
         const StepPlan sp = plan_step(st, reduced(L));
@@ -1137,7 +1138,7 @@ klb_status build_tables(klb_batch *B, int width)
     const int n = (int)B->mem.size(), P = B->period;
     std::vector<int> &prefix = B->prefix;
     B->table.resize((size_t)P * n * B->rec_size);
-    B->ck.resize(3 * (size_t)n);
+    B->ck.resize(n);
     prefix.assign(n + 1, 0);
     B->plans.resize((size_t)P * n);
     B->acc.assign(P, 0);
@@ -1157,6 +1158,9 @@ klb_status build_tables(klb_batch *B, int width)
         KLB_BCUDA(B, cudaMemcpy(B->base + B->table_off, B->table.data(), B->table.size(), cudaMemcpyHostToDevice));
         KLB_BCUDA(B, cudaMemcpy(B->base + B->prefix_off, prefix.data(), prefix.size() * sizeof(int),
                                 cudaMemcpyHostToDevice));
+        if (B->storage != KLB_FP64)
+            KLB_BCUDA(B, cudaMemcpy(B->base + B->ck_off, B->ck.data(), B->ck.size() * sizeof(CollideSet),
+                                    cudaMemcpyHostToDevice));
     }
     KLB_BCUDA(B, cudaMemset(B->base + B->reps_off, 0, sizeof(uint32_t)));
     B->width = width;
@@ -1192,7 +1196,8 @@ cudaError_t launch_phase(klb_batch *B, int k)
     }
     const size_t at = (size_t)k * n * B->rec_size;
     const BatchLaunch b{B->table.data() + at, B->base + B->table_off + at, B->prefix.data(),
-                        (const int *)(B->base + B->prefix_off), B->ck.data(), (int)n, B->width, B->acc[k] != 0, B->ep, B->by_table};
+                        (const int *)(B->base + B->prefix_off), B->ck.data(),
+                        (const CollideSet *)(B->base + B->ck_off), (int)n, B->width, B->acc[k] != 0, B->ep, B->by_table};
     cudaError_t e = launch_batch(B->Q, B->storage, b, B->stream);
     if (e == cudaSuccess && k == B->period - 1) e = launch_count_period((uint32_t *)(B->base + B->reps_off), B->stream);
     return e;
@@ -1304,8 +1309,8 @@ klb_status run_steps(klb_batch *B, int64_t nsteps, bool use_graph)
 
 size_t klb::batch_table_bytes(int storage, int n)
 {
-    size_t t, p, r;
-    return n < 1 ? 0 : batch_layout(n, storage, &t, &p, &r);
+    size_t t, p, c, r;
+    return n < 1 ? 0 : batch_layout(n, storage, &t, &p, &c, &r);
 }
 
 extern "C" {
@@ -1313,8 +1318,8 @@ extern "C" {
 size_t klb_batch_bytes(klb_lattice *const *members, int n)
 {
     if (!members || n < 1 || !members[0]) return 0;
-    size_t t, p, r;
-    return batch_layout(n, members[0]->desc.storage, &t, &p, &r);
+    size_t t, p, c, r;
+    return batch_layout(n, members[0]->desc.storage, &t, &p, &c, &r);
 }
 
 klb_status klb_batch_create(klb_lattice *const *members, int n, void *dev_buf, size_t bytes,
@@ -1342,7 +1347,7 @@ klb_status klb_batch_create(klb_lattice *const *members, int n, void *dev_buf, s
     B->storage = members[0]->desc.storage;
     B->period = batch_period(B->storage);
     B->rec_size = rec_size(B->storage);
-    const size_t need = batch_layout(n, B->storage, &B->table_off, &B->prefix_off, &B->reps_off);
+    const size_t need = batch_layout(n, B->storage, &B->table_off, &B->prefix_off, &B->ck_off, &B->reps_off);
     if (!dev_buf || ((uintptr_t)dev_buf & 255u)) {
         delete B;
         return fail(nullptr, KLB_EINVAL, "dev_buf must be a 256-byte aligned device pointer");

@@ -202,6 +202,11 @@ inline __host__ __device__ CollideK collide_k(int Q, float om)
     return c;
 }
 
+// The constants of a lattice's three species.
+struct alignas(16) CollideSet {
+    CollideK s[3];
+};
+
 // What a step reads of its lattice: the record that a batch keeps per phase
 // and member.  T is the arithmetic type (float or double); the populations
 // are stored as T, or as FP16/BF16 against per-row references.
@@ -245,7 +250,7 @@ struct alignas(16) StepRecord {
 // and formed from it, and what the other passes read.
 template <typename T>
 struct alignas(16) StepArgs : StepRecord<T> {
-    CollideK ck[3];          // FP32 arithmetic: collision constants per species
+    CollideSet ck;           // FP32 arithmetic: collision constants
     const void *in_prev[3];  // observe mode: previous state and its references (residual),
     const float *dec_prev[3];
     const T *U3[2];          // u(n-3),
@@ -278,19 +283,19 @@ cudaError_t launch_finalize(const double *partials, int nblocks, double *sums, c
 // One more period completed by a batch (StepArgs::step_reps).
 cudaError_t launch_count_period(uint32_t *reps, cudaStream_t s);
 // One step of many lattices: argument records and first block of each lattice
-// (prefix[n] = total blocks), and the collision constants, three per lattice.
+// (prefix[n] = total blocks), and the collision constants.
 // Up to kBatchParams records go as kernel parameters (32 KB in all).  More
 // lattices take several such launches, or one over device copies of the
 // records (batch_by_table).  A launch waits for the one before it, so several
 // pay only when each fills the chip (20 warps on each of 152 SMs) some times
 // over: kGroupItems items (warps) in each.  One launch -> several, us per
 // step, GB300, FP32 / FP16, by items per launch: 1333 (400 D2Q9 slabs 64x40)
-// 24.7 -> 57.0 / 72.2 -> 104; 4466 (400 pipes R 4-5, nx 3) 145 -> 165 / 229 ->
-// 245; 4824 (72 of them) 25.9 -> 26.1 / 36.2 -> 39.0; 7020 (40 pipes R 6-9, nx
-// 8) 35.6 -> 35.3 / 42.4 -> 42.9; 9065 (40 sweep channels at a quarter) 44.1 ->
-// 43.0 / 49.2 -> 49.3; 11700 (100 pipes R 6-9) 87.9 -> 83.0 / 117 -> 113;
-// 61200 (40 channels at half) 232 -> 214 / 238 -> 219.  FP64, which the FP64
-// pipe bounds, takes one launch throughout (61200: 427 -> 450 at a quarter).
+// 24.2 -> 56.4 / 70.5 -> 102; 4466 (400 pipes R 4-5, nx 3) 141 -> 166 / 223 ->
+// 243; 4824 (72 of them) 24.8 -> 26.1 / 36.3 -> 38.8; 7020 (40 pipes R 6-9, nx
+// 8) 34.8 -> 35.0 / 41.5 -> 42.9; 9065 (40 sweep channels at a quarter) 44.0 ->
+// 43.1 / 48.6 -> 49.2; 11700 (100 pipes R 6-9) 85.6 -> 82.6 / 115 -> 112;
+// 61200 (40 channels at half) 232 -> 214 / 234 -> 218.  FP64, which the FP64
+// pipe bounds, takes one launch throughout (9065: 428 -> 451).
 constexpr int kBatchParams = 36;
 constexpr long long kGroupItems = 8000;
 inline int batch_groups(int n) { return (n + kBatchParams - 1) / kBatchParams; }
@@ -301,7 +306,7 @@ inline bool batch_by_table(int n, int storage, long long items)
 struct BatchLaunch {
     const void *table, *dev_table;
     const int *prefix, *dev_prefix;
-    const CollideK *ck;
+    const CollideSet *ck, *dev_ck;
     int n, width;
     bool acc, ep, by_table;
 };

@@ -1092,20 +1092,21 @@ cudaError_t launch_step(void (*kernel)(A), int nblocks, int bx, cudaStream_t s, 
 // arguments.
 template <int Q, typename T, typename S, bool ACC, bool EP>
 __global__ void __launch_bounds__(kBlockX, (step_min_blocks<T, S, EP>()))
-    k_step_batch(const StepRecord<T> *__restrict__ table, const int *__restrict__ prefix, int n)
+    k_step_batch(const StepRecord<T> *__restrict__ table, const CollideSet *__restrict__ ck,
+                 const int *__restrict__ prefix, int n)
 {
     pdl_launch_dependents();
     __shared__ StepArgs<T> sp;
     int c = 0;
     for (int m = 1 + ((int)threadIdx.x & 31); m < n; m += 32) c += __ldg(prefix + m) <= (int)blockIdx.x;
     const int lid = (int)__reduce_add_sync(0xffffffffu, (unsigned)c);
-    static_assert(sizeof(StepRecord<T>) % 16 == 0, "argument record in 16-byte words");
-    const int4 *src = reinterpret_cast<const int4 *>(table + lid);
-    int4 *dst = reinterpret_cast<int4 *>(static_cast<StepRecord<T> *>(&sp));
-    for (int k = threadIdx.x; k < (int)(sizeof(StepRecord<T>) / 16); k += blockDim.x) dst[k] = __ldg(src + k);
-    if constexpr (sizeof(T) == 4) {
-        if (threadIdx.x < 3) sp.ck[threadIdx.x] = collide_k(Q, __ldg(&table[lid].om[threadIdx.x]));
-    }
+    // record and constants in one round of loads (two rounds, or the constants
+    // formed here, cost up to 5% of a step of small channels)
+    static_assert(sizeof(StepRecord<T>) % 16 == 0 && sizeof(CollideSet) % 16 == 0, "16-byte words");
+    constexpr int NR = (int)(sizeof(StepRecord<T>) / 16), NC = sizeof(T) == 4 ? (int)(sizeof(CollideSet) / 16) : 0;
+    const int4 *src = reinterpret_cast<const int4 *>(table + lid), *csrc = reinterpret_cast<const int4 *>(ck + lid) - NR;
+    int4 *dst = reinterpret_cast<int4 *>(static_cast<StepRecord<T> *>(&sp)), *cdst = reinterpret_cast<int4 *>(&sp.ck) - NR;
+    for (int k = threadIdx.x; k < NR + NC; k += blockDim.x) (k < NR ? dst : cdst)[k] = __ldg((k < NR ? src : csrc) + k);
     __syncthreads();
     step_cells_body<Q, T, S, ACC, false, EP>(sp, (int)blockIdx.x - __ldg(prefix + lid));
 }
@@ -1262,7 +1263,7 @@ cudaError_t launch_batch_form(const BatchLaunch &b, cudaStream_t s)
     if (b.by_table) {
         cfg.gridDim = dim3((unsigned)b.prefix[b.n]);
         return cudaLaunchKernelEx(&cfg, k_step_batch<Q, T, S, ACC, EP>, static_cast<const StepRecord<T> *>(b.dev_table),
-                                  b.dev_prefix, b.n);
+                                  b.dev_ck, b.dev_prefix, b.n);
     }
     const int groups = batch_groups(b.n);
     for (int g = 0; g < groups; ++g) {
@@ -1271,7 +1272,7 @@ cudaError_t launch_batch_form(const BatchLaunch &b, cudaStream_t s)
         tb.n = m1 - m0;
         for (int m = m0; m < m1; ++m) {
             static_cast<StepRecord<T> &>(tb.a[m - m0]) = static_cast<const StepRecord<T> *>(b.table)[m];
-            for (int s = 0; s < 3; ++s) tb.a[m - m0].ck[s] = b.ck[3 * m + s];
+            tb.a[m - m0].ck = b.ck[m];
         }
         for (int m = m0; m <= m1; ++m) tb.prefix[m - m0] = b.prefix[m] - b.prefix[m0];
         cfg.gridDim = dim3((unsigned)tb.prefix[tb.n]);

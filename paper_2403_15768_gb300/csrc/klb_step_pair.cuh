@@ -709,7 +709,7 @@ __device__ __forceinline__ void step_body2(const StepArgs<float> &p, int b)
         if constexpr (NOISE)
             return collide_k(Q, p.om[s]);
         else
-            return p.ck[s];
+            return p.ck.s[s];
     };
     if (water) {
         float2 g[Q], j[3];
