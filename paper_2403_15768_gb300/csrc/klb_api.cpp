@@ -119,9 +119,10 @@ void fill_level(const klb_lattice *L, const HostState &st, StepArgs<T> &a)
 }
 
 // All kernel arguments for the time level `st`; the step kernel runs blocks
-// of sbx threads and touches all_bytes of state buffers per launch.
+// of sbx threads, with the small-lattice form of the solid rows or not, and
+// touches all_bytes of state buffers per launch.
 template <typename T>
-void fill_args_at(const klb_lattice *L, const HostState &st, int sbx, bool ep, size_t all_bytes, StepArgs<T> &a)
+void fill_args_at(const klb_lattice *L, const HostState &st, int sbx, bool fine, size_t all_bytes, StepArgs<T> &a)
 {
     const Geometry &g = L->geo;
     const MemoryPlan &p = L->plan;
@@ -144,7 +145,7 @@ void fill_args_at(const klb_lattice *L, const HostState &st, int sbx, bool ep, s
     a.nchunk = p.nchunk;
     a.nbw = (int)g.rows[kFluid].size() * a.nchunk;
     a.snchunk = (g.nx + sbx - 1) / sbx;
-    a.split = L->desc.storage == KLB_FP64 && fp64_split(g.nx, a.n_rows[kFluid], a.n_rows[kSolid]);
+    a.split = L->desc.storage == KLB_FP64 && fine;
     // divisions by multiplication: the kernel's first instructions wait for them
     auto divider = [](int d, uint32_t &mul, uint32_t &shift) {
         uint32_t sh = 0;
@@ -153,7 +154,7 @@ void fill_args_at(const klb_lattice *L, const HostState &st, int sbx, bool ep, s
         mul = (uint32_t)((1ull << (31 + sh)) / (uint32_t)d + 1);
     };
     a.nseg64 = (g.nx + 63) / 64;
-    a.sseg = ep ? (g.nx + 31) / 32 : a.nseg64;
+    a.sseg = fine ? (g.nx + 31) / 32 : a.nseg64;
     divider(a.nseg64, a.seg_mul, a.seg_shift);
     divider(a.sseg, a.sseg_mul, a.sseg_shift);
     a.nch32 = (g.nx + 31) / 32;
@@ -184,7 +185,7 @@ void fill_args_at(const klb_lattice *L, const HostState &st, int sbx, bool ep, s
 template <typename T>
 void fill_args(const klb_lattice *L, StepArgs<T> &a)
 {
-    fill_args_at(L, L->st, L->plan.sbx, L->plan.ep, state_bytes(L), a);
+    fill_args_at(L, L->st, L->plan.sbx, L->plan.fine, state_bytes(L), a);
 }
 
 // The host side of one step: encode generation of the output, whether the
@@ -690,7 +691,8 @@ klb_status klb_step(klb_lattice *L, int64_t nsteps)
         cudaError_t e = with_args(L, [&](void *a) {
             set_enc(L, a, sp.outgen);
             const int mode = sp.acc ? kModeStepAcc : (L->kT > 0.0 ? kModeStepNoise : kModeStep);
-            return launch(L->geo.Q, L->desc.storage, a, L->plan.ep ? mode | kModeEp : mode, L->plan.snblocks, L->plan.sbx, L->stream);
+            const bool ep = L->plan.fine && L->desc.storage != KLB_FP64;
+            return launch(L->geo.Q, L->desc.storage, a, ep ? mode | kModeEp : mode, L->plan.snblocks, L->plan.sbx, L->stream);
         });
         if (e != cudaSuccess) return cuda_fail(L, e, "step kernel launch");
         advance(L->st, sp);
@@ -1049,7 +1051,7 @@ struct klb_batch {
     int period = 6;
     int width = kBlockX;
     int nblocks = 0;
-    bool ep = false, by_table = false;
+    bool fine = false, by_table = false;  // small-lattice form of the solid rows; launched over device copies
     size_t rec_size = 0, table_off = 0, prefix_off = 0, ck_off = 0, reps_off = 0;
     std::vector<char> table;      // argument records [phase][member], the block prefix
     std::vector<int> prefix;
@@ -1103,6 +1105,13 @@ void destroy_graph(klb_batch *B)
     B->graph = nullptr;
 }
 
+// Whether the solid rows of a member take the small-lattice form: with FP32
+// arithmetic one form for the launch, with FP64 the members that take it alone.
+bool fine_member(const klb_batch *B, const klb_lattice *L)
+{
+    return B->fine && (B->storage != KLB_FP64 || L->plan.fine);
+}
+
 // A member's argument records of every phase, from its time level now: the
 // arguments once, then what follows the time level.
 template <typename T>
@@ -1111,7 +1120,7 @@ void fill_records(klb_batch *B, int m, int width, size_t all_bytes)
     const klb_lattice *L = B->mem[m];
     const int n = (int)B->mem.size(), P = B->period;
     StepArgs<T> a;
-    fill_args_at(L, L->st, width, B->ep, all_bytes, a);
+    fill_args_at(L, L->st, width, fine_member(B, L), all_bytes, a);
     a.step_reps = (const uint32_t *)(B->base + B->reps_off);
     a.step_period = P;
     B->ck[m] = a.ck;
@@ -1151,7 +1160,7 @@ klb_status build_tables(klb_batch *B, int width)
             fill_records<float>(B, m, width, all_bytes);
         const Geometry &g = B->mem[m]->geo;
         prefix[m + 1] = prefix[m] + step_blocks(g.nx, (int)g.rows[kFluid].size(), (int)g.rows[kSolid].size(), width,
-                                                B->storage, B->ep);
+                                                B->storage, fine_member(B, B->mem[m]));
     }
     KLB_BCUDA(B, cudaStreamSynchronize(B->stream));
     if (B->by_table) {
@@ -1197,7 +1206,8 @@ cudaError_t launch_phase(klb_batch *B, int k)
     const size_t at = (size_t)k * n * B->rec_size;
     const BatchLaunch b{B->table.data() + at, B->base + B->table_off + at, B->prefix.data(),
                         (const int *)(B->base + B->prefix_off), B->ck.data(),
-                        (const CollideSet *)(B->base + B->ck_off), (int)n, B->width, B->acc[k] != 0, B->ep, B->by_table};
+                        (const CollideSet *)(B->base + B->ck_off), (int)n, B->width, B->acc[k] != 0,
+                        B->fine && B->storage != KLB_FP64, B->by_table};
     cudaError_t e = launch_batch(B->Q, B->storage, b, B->stream);
     if (e == cudaSuccess && k == B->period - 1) e = launch_count_period((uint32_t *)(B->base + B->reps_off), B->stream);
     return e;
@@ -1369,18 +1379,21 @@ klb_status klb_batch_create(klb_lattice *const *members, int n, void *dev_buf, s
         return fail(nullptr, KLB_ECUDA, m);
     }
     int w = kBlockX;
-    long long items[2] = {0, 0};
+    long long items[2] = {0, 0}, warps64 = 0;
     for (klb_lattice *L : B->mem) {
         const Geometry &g = L->geo;
-        for (int e = 0; e < 2; ++e) items[e] += step_items(g.nx, g.rows[kFluid].size(), g.rows[kSolid].size(), e != 0);
+        const long long nw = (long long)g.rows[kFluid].size(), ns = (long long)g.rows[kSolid].size();
+        for (int e = 0; e < 2; ++e) items[e] += step_items(g.nx, nw, ns, e != 0);
+        warps64 += fp64_warps(g.nx, nw, ns);
     }
     if (B->storage == KLB_FP64) {
-        for (klb_lattice *L : B->mem) w = std::min(w, L->plan.sbx);
+        B->fine = fp64_batch_split(warps64);
+        for (klb_lattice *L : B->mem) w = std::min(w, B->fine ? L->plan.sbx : L->plan.bx);
     } else {
-        B->ep = step_ep(items[1]);
-        w = step_width(items[B->ep]);
+        B->fine = step_ep(items[1]);
+        w = step_width(items[B->fine]);
     }
-    B->by_table = batch_by_table(n, B->storage, items[B->ep]);
+    B->by_table = batch_by_table(n, B->storage, items[B->fine]);
     klb_status st = build_tables(B, w);
     if (st != KLB_OK) {
         std::string m = B->err;

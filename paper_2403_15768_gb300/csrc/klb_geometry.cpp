@@ -353,16 +353,16 @@ MemoryPlan plan_memory(const Geometry &g, int storage)
     p.nchunk = (g.nx + p.bx - 1) / p.bx;
     p.nblocks_w = (int)nr[kFluid] * p.nchunk;
     p.nblocks_s = (int)nr[kSolid] * p.nchunk;
-    p.ep = false;
     if (storage == KLB_FP64) {
-        p.sbx = fp64_split(g.nx, (int)nr[kFluid], (int)nr[kSolid]) ? 32 : p.bx;
+        p.fine = fp64_split(g.nx, (int)nr[kFluid], (int)nr[kSolid]);
+        p.sbx = p.fine ? 32 : p.bx;
         p.static_blocks = p.nblocks_w + p.nblocks_s;
     } else {
-        p.ep = step_ep(step_items(g.nx, nr[kFluid], nr[kSolid], true));
-        p.sbx = step_width(step_items(g.nx, nr[kFluid], nr[kSolid], p.ep));
+        p.fine = step_ep(step_items(g.nx, nr[kFluid], nr[kSolid], true));
+        p.sbx = step_width(step_items(g.nx, nr[kFluid], nr[kSolid], p.fine));
         p.static_blocks = (int)(nr[kFluid] + nr[kSolid]) * ((g.nx + 255) / 256);
     }
-    p.snblocks = step_blocks(g.nx, (int)nr[kFluid], (int)nr[kSolid], p.sbx, storage, p.ep);
+    p.snblocks = step_blocks(g.nx, (int)nr[kFluid], (int)nr[kSolid], p.sbx, storage, p.fine);
     {
         // Observation grid: at most the 4 blocks of 4 warps that fit an SM at
         // 128 registers, no more blocks than items (64 cells of a row) need,

@@ -97,7 +97,7 @@ struct MemoryPlan {
     size_t bounds;         // error word of debug builds (KLB_BOUNDS)
     size_t total;
     int nblocks_w, nblocks_s, nchunk, bx;  // one cell per thread (observe, field, init)
-    bool ep;                               // step kernel: form of the solid items (step_ep),
+    bool fine;                             // step kernel: small-lattice form of the solid rows (step_ep, fp64_split),
     int sbx, snblocks;                     // threads per block, blocks
     int static_blocks;                     // row chunks that klb_observables_static bounds
     int oblocks, oblocks_s;                // observation with FP32 arithmetic: blocks of kBlockX, of which solid
@@ -116,20 +116,25 @@ constexpr float kFp16Scale = 1048576.0f;  // 2^20
 // blocks leaves SMs idle: one warp per block, and solid rows one species per
 // block.  The FP64 pipe takes 16 cycles per warp instruction on every SM, so
 // a step lasts as long as its busiest SM computes.
-inline bool fp64_split(int nx, int rows_w, int rows_s)
-{
-    return ((long long)rows_w + 2LL * rows_s) * ((nx + 31) / 32) <= 152;
-}
+inline long long fp64_warps(int nx, long long rows_w, long long rows_s) { return (rows_w + 2 * rows_s) * ((nx + 31) / 32); }
+inline bool fp64_split(int nx, int rows_w, int rows_s) { return fp64_warps(nx, rows_w, rows_s) <= 152; }
+
+// Whether the members of a batch (warps: fp64_warps of all) keep that form:
+// while all of them find a place on the chip (16 warps on each of 152 SMs).
+// Beyond, the second species streamed and collided for nothing is what the
+// FP64 pipe waits for.  Step times with -> without, GB300: 24 slabs of 64x40
+// (2304 warps) 24.3 -> 27.9 us, 36 (3456) 34.1 -> 33.4, 100 75.5 -> 70.6, 400
+// 273 -> 242; 400 slabs of 16x20 (10400) 87.3 -> 77.8.
+inline bool fp64_batch_split(long long warps) { return warps <= 152 * 16; }
 
 // Blocks of sbx threads of one step launch: FP64 one block per row chunk of
-// sbx cells (a solid one per species with fp64_split); FP32 arithmetic one warp per item of 64 cells (two adjacent x
-// per thread, packed f32x2).
+// sbx cells (with `fine` a solid one per species, fp64_split); FP32 arithmetic
+// one warp per item (`fine`: species pairs, step_ep).
 inline long long step_items(int nx, long long rows_w, long long rows_s, bool ep);
-inline int step_blocks(int nx, int rows_w, int rows_s, int sbx, int storage, bool ep)
+inline int step_blocks(int nx, int rows_w, int rows_s, int sbx, int storage, bool fine)
 {
-    if (storage == KLB_FP64)
-        return (rows_w + rows_s + (fp64_split(nx, rows_w, rows_s) ? rows_s : 0)) * ((nx + sbx - 1) / sbx);
-    return (int)((step_items(nx, rows_w, rows_s, ep) + sbx / 32 - 1) / (sbx / 32));
+    if (storage == KLB_FP64) return (rows_w + rows_s + (fine ? rows_s : 0)) * ((nx + sbx - 1) / sbx);
+    return (int)((step_items(nx, rows_w, rows_s, fine) + sbx / 32 - 1) / (sbx / 32));
 }
 
 // Items of one launch of the FP32-arithmetic step on a lattice's rows: 64
@@ -308,7 +313,7 @@ struct BatchLaunch {
     const int *prefix, *dev_prefix;
     const CollideSet *ck, *dev_ck;
     int n, width;
-    bool acc, ep, by_table;
+    bool acc, ep, by_table;  // ep: species pairs (FP32 arithmetic)
 };
 cudaError_t launch_batch(int Q, int storage, const BatchLaunch &b, cudaStream_t s);
 

@@ -42,3 +42,20 @@ def test_table_launch_matches_stepping_alone(base, nx, n, storage):
         alone[k].step(39 + 9 + 31)
         for a, b in zip(alone[k].get_state(), mates[k].get_state()):
             assert np.array_equal(a, b), k
+
+
+@pytest.mark.parametrize("n", [3, 25, 26])
+def test_fp64_batch_form_matches_stepping_alone(n):
+    """FP64 slabs of 96 warps that alone keep one species per solid block: in a batch as long as all its
+    warps fit the chip (25 members), both species per block beyond."""
+    w = SLAB9.with_(nx=64, ny=40, width=32, shell=4, storage="fp64")
+    mates, alone = [klb.lattice_from_workload(w) for _ in range(n)], klb.lattice_from_workload(w)
+    for lat in (mates[0], mates[-1], alone):
+        lat.init_equilibrium(*inputs.perturbation(w, 4, 1e-3))
+    batch = klb.Batch(mates)
+    assert (batch.blocks == n * (32 + 16) * 2) == (n <= 25)
+    batch.step(25)
+    alone.step(25)
+    for lat in (mates[0], mates[-1]):
+        for a, b in zip(alone.get_state(), lat.get_state()):
+            assert np.array_equal(a, b)
