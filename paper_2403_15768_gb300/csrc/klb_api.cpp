@@ -871,16 +871,25 @@ klb_status klb_set_state(klb_lattice *L, const double *gin, const double *U1, co
     const float scale = storage == KLB_FP16_DEV ? kFp16Scale : 1.0f;
     auto sat = [](float v, float m) { return v > m ? m : (v < -m ? -m : v); };  // NaN passes
     KLB_CUDA(L, cudaStreamSynchronize(L->stream));
-    reset_state(L, step);
-    std::vector<float> enc[3], dec[3];
-    HostBuf pops, Us[2];
+    // All host memory first: without it the state and its time level stay as they are.
+    HostBuf encs[3], decs[3], pops, Us[2];
     StreamGuard guard{L->stream};
     const MemoryPlan &p = L->plan;
-    if (!pops.alloc(pops_bytes(L))) return no_host_memory(L);
+    bool have = pops.alloc(pops_bytes(L));
+    for (int t = 0; t < 2; ++t) have = have && Us[t].alloc(p.U[0][1] - p.U[0][0] + p.U_bytes[kSolid]);
+    for (int s = 0; red && s < 3; ++s) have = have && encs[s].alloc(p.ref_bytes[s]) && decs[s].alloc(p.ref_bytes[s]);
+    if (!have) return no_host_memory(L);
+    reset_state(L, step);
+    float *enc[3] = {}, *dec[3] = {};
+    for (int s = 0; red && s < 3; ++s) {
+        enc[s] = encs[s].as<float>();
+        dec[s] = decs[s].as<float>();
+        std::memset(enc[s], 0, p.ref_bytes[s]);
+        std::memset(dec[s], 0, p.ref_bytes[s]);
+    }
     for (int s = 0; s < 3; ++s) {
         const int c = cls_of(s);
         const size_t nr = g.rows[c].size();
-        if (red) enc[s].assign(nr * kRefStride, 0.f);
         auto take = [&](auto *pop) {
             using V = std::decay_t<decltype(*pop)>;
             host_parallel((size_t)Q * nr, (size_t)Q * nr * nx * sizeof(double), [&, pop, nr, s, c](size_t k0, size_t k1) {
@@ -930,23 +939,21 @@ klb_status klb_set_state(klb_lattice *L, const double *gin, const double *U1, co
         for (int s = 0; s < 3; ++s) {
             const int c = cls_of(s);
             const size_t nr = g.rows[c].size();
-            dec[s].assign(nr * kRefStride, 0.f);
             for (size_t r = 0; r < nr; ++r)
                 for (int i = 0; i < Q; ++i) {
                     const long q = g.info[c][r].src[i] / (g.nxp / kRowAlign);  // sdir * nr + srow
                     const long sdir = q / (long)nr, srow = q - sdir * (long)nr;
                     dec[s][r * kRefStride + i] = enc[s][srow * kRefStride + sdir];
                 }
-            KLB_CUDA(L, cudaMemcpyAsync(dev(L, L->plan.ref_enc[0][s]), enc[s].data(), L->plan.ref_bytes[s],
+            KLB_CUDA(L, cudaMemcpyAsync(dev(L, L->plan.ref_enc[0][s]), enc[s], L->plan.ref_bytes[s],
                                         cudaMemcpyHostToDevice, L->stream));
-            KLB_CUDA(L, cudaMemcpyAsync(dev(L, L->plan.ref_dec[0][s]), dec[s].data(), L->plan.ref_bytes[s],
+            KLB_CUDA(L, cudaMemcpyAsync(dev(L, L->plan.ref_dec[0][s]), dec[s], L->plan.ref_bytes[s],
                                         cudaMemcpyHostToDevice, L->stream));
         }
     }
     const double *Ui[2] = {U1, U2};  // u(n-1), u(n-2)
     for (int t = 0; t < 2; ++t) {
-        const size_t *at = p.U[slot_of(step - 1 - t)], n = at[1] - at[0] + p.U_bytes[kSolid];
-        if (!Us[t].alloc(n)) return no_host_memory(L);
+        const size_t *at = p.U[slot_of(step - 1 - t)], n = Us[t].bytes;
         for (int c = 0; c < 2; ++c) {
             const size_t ns = g.slot_row[c].size();
             if (!ns) continue;
