@@ -181,10 +181,31 @@ void fill_args_at(const klb_lattice *L, const HostState &st, int sbx, bool fine,
     a.ahead = step_ahead(g.Q, d.storage, g.nxp, all_bytes);
 }
 
+// Form of the solid rows, threads per block and blocks of a lattice's step:
+// those of its plan, but for thermal noise in FP32, which has its own rule.
+struct StepForm {
+    bool fine;
+    int sbx, blocks;
+};
+
+StepForm step_form(const klb_lattice *L)
+{
+    const Geometry &g = L->geo;
+    const long long nw = (long long)g.rows[kFluid].size(), ns = (long long)g.rows[kSolid].size();
+    StepForm f{L->plan.fine, L->plan.sbx, L->plan.snblocks};
+    if (L->kT > 0.0 && f.fine && L->desc.storage == KLB_FP32 && !noise_ep(g.Q, step_items(g.nx, nw, ns, true))) {
+        f.fine = false;
+        f.sbx = step_width(step_items(g.nx, nw, ns, false));
+        f.blocks = step_blocks(g.nx, (int)nw, (int)ns, f.sbx, KLB_FP32, false);
+    }
+    return f;
+}
+
 template <typename T>
 void fill_args(const klb_lattice *L, StepArgs<T> &a)
 {
-    fill_args_at(L, L->st, L->plan.sbx, L->plan.fine, state_bytes(L), a);
+    const StepForm f = step_form(L);
+    fill_args_at(L, L->st, f.sbx, f.fine, state_bytes(L), a);
 }
 
 // The host side of one step: encode generation of the output, whether the
@@ -660,8 +681,9 @@ klb_status klb_step(klb_lattice *L, int64_t nsteps)
         cudaError_t e = with_args(L, [&](void *a) {
             set_enc(L, a, sp.outgen);
             const int mode = sp.acc ? kModeStepAcc : (L->kT > 0.0 ? kModeStepNoise : kModeStep);
-            const bool ep = L->plan.fine && L->desc.storage != KLB_FP64;
-            return launch(L->geo.Q, L->desc.storage, a, ep ? mode | kModeEp : mode, L->plan.snblocks, L->plan.sbx, L->stream);
+            const StepForm f = step_form(L);
+            const bool ep = f.fine && L->desc.storage != KLB_FP64;
+            return launch(L->geo.Q, L->desc.storage, a, ep ? mode | kModeEp : mode, f.blocks, f.sbx, L->stream);
         });
         if (e != cudaSuccess) return cuda_fail(L, e, "step kernel launch");
         advance(L->st, sp);
@@ -710,8 +732,8 @@ klb_status klb_observables_static(klb_lattice *L, klb_obs *out)
     KLB_CUDA(L, static_scratch(&partials, &sums, &max_blocks));
     if ((size_t)static_blocks(L) > max_blocks)
         return fail(L, KLB_EINVAL,
-                    "observation pass needs " + std::to_string(static_blocks(L)) +
-                        " blocks, more than the static scratch holds (KLB_STATIC_MAX_BLOCKS = " +
+                    std::to_string(static_blocks(L)) +
+                        " row chunks, more than the static observation takes (KLB_STATIC_MAX_BLOCKS = " +
                         std::to_string(max_blocks) + ")");
     KLB_CUDA(L, launch_observe(L, partials, sums));
     double S[kNumSums];

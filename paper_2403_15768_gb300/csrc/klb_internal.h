@@ -152,11 +152,24 @@ inline long long step_items(int nx, long long rows_w, long long rows_s, bool ep)
 // GB300, FP32: pipe R 8, nx 8 (384 items) 5.6 -> 3.8 us, nx 200 7.7 -> 5.5,
 // nx 400 (3792 items) 9.5 -> 7.7; 128x64x64 (5552 items) 8.5 -> 8.8; R 48,
 // nx 8 (9176 items) 11.0 -> 11.3; 512x128x128 134.9 -> 140.9.
+// FP16: 384 items 5.9 -> 4.2 us, 3160 9.4 -> 7.0, 3576 8.6 -> 7.4, 3812 7.3 ->
+// 7.6.
 inline bool step_ep(long long ep_items) { return ep_items <= 4000; }
 
+// The same with thermal noise, whose water cells take most of the time: on
+// D3Q19 while nearly all items find a place at once (16 warps of 128 registers
+// on each of 152 SMs), on D2Q9 never.  Cell pairs -> species pairs: 764 items
+// 9.0 -> 6.8 us, 2424 10.0 -> 7.8, 2612 10.4 -> 9.0, 2780 9.6 -> 9.7, 2872 10.0
+// -> 9.9, 3024 9.3 -> 10.8, 3232 10.1 -> 9.9, 3576 9.5 -> 11.2; D2Q9 48 to 420
+// items equal, 1100 5.1 -> 5.5, 1600 4.9 -> 5.7.
+inline bool noise_ep(int Q, long long ep_items) { return Q == 19 && ep_items <= 2900; }
+
 // Threads per step block with FP32 arithmetic: four warps, or one where the
-// launch's items fit the chip at once anyway (20 warps on each of 152 SMs),
-// which spreads them over all SMs.
+// launch's items are few, which spreads them over all SMs (20 warps of cell
+// pairs, 16 of species pairs find a place on each of 152 SMs).  For species
+// pairs the width matters little: four -> one, FP32 1616 items 5.70 -> 5.62 us,
+// 2592 6.25 -> 6.24, 3160 6.69 -> 6.81; FP16 5.54 -> 5.58, 6.48 -> 6.51, 6.95 ->
+// 7.07.
 inline int step_width(long long items) { return items <= 152 * 20 ? 32 : kBlockX; }
 
 inline bool reduced_storage(int storage) { return storage == KLB_FP16_DEV || storage == KLB_BF16_DEV; }

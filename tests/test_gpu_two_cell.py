@@ -102,6 +102,27 @@ def test_noise_on_two_cells_matches_the_oracle(nx, change):
         assert np.abs(dg - dr).max() <= 2e-4 * max(np.abs(dr).max(), 1e-12), s
 
 
+@pytest.mark.parametrize("w", [PIPE.with_(nx=128, ny=42, nz=42, radius=15), PIPE.with_(nx=101, ny=42, nz=42, radius=15, **WAVES),
+                               inputs.SLAB_D2Q9_FP64.with_(nx=65, ny=60, width=40, shell=10, storage="fp32")],
+                         ids=["specular", "waves", "d2q9"])
+def test_noise_where_only_the_noise_free_step_takes_species_pairs(w):
+    """Noise off, on and off again on lattices of up to 4000 items whose noisy steps take two cells."""
+    o, lat = make_oracle(w), klb.lattice_from_workload(w)
+    assert not _takes_two_cells(lat, w)
+    o.init_equilibrium()
+    for steps, kT in ((2, 0.0), (7, 1e-5), (3, 0.0)):
+        o.set_fluctuations(kT, 99)
+        lat.set_fluctuations(kT, 99)
+        o.step(steps)
+        lat.step(steps)
+    f, (drho, u) = o.observe(), lat.get_field()
+    for s, m in enumerate(species_masks(o.geo, w.nx)):
+        ref, got = f["u"][s][:, m], u[s][:, m]
+        assert np.abs(got - ref).max() <= 2e-4 * np.abs(ref).max(), s
+        dr, dg = f["drho"][s][m], drho[s][m]
+        assert np.abs(dg - dr).max() <= 2e-4 * max(np.abs(dr).max(), 1e-12), s
+
+
 @pytest.mark.parametrize("storage", ["fp32", "fp16", "bf16"])
 def test_requests_to_l2_change_no_bits(storage):
     """Lattices below the 129 MB L2 that alone ask it for nothing, in a batch beyond it that does."""
