@@ -335,6 +335,25 @@ struct StreamGuard {
 
 klb_status no_host_memory(klb_lattice *L) { return fail(L, KLB_ENOMEM, "host allocation failed"); }
 
+// n rows of nx elements padded to nxp: fill(k, o) writes row k's elements, the
+// padding is zeroed here.  Where padding is a fifth of a row or more, all rows
+// at once beforehand: lines of memory that the device has read are slow to
+// write in parts, and a call per row takes longer than a narrow row's elements
+// (150x150 pipe, nx 5: klb_init_equilibrium FP32 1.9 to 3.7 -> 0.56 ms, FP64 4.0
+// to 7.5 -> 1.15; pipe R8, nx 8: klb_set_state FP64 0.26 to 0.42 -> 0.19 ms).
+template <typename V, typename F>
+void fill_rows(V *rows, size_t n, size_t nx, size_t nxp, F fill)
+{
+    const bool narrow = nx < 4 * (nxp - nx);
+    if (narrow) std::memset((void *)rows, 0, n * nxp * sizeof(V));
+    for (size_t k = 0; k < n; ++k) {
+        V *o = rows + k * nxp;
+        fill(k, o);
+        if (!narrow)
+            for (size_t x = nx; x < nxp; ++x) o[x] = V(0);
+    }
+}
+
 // Rows of host box fields (either may be null) in the layout of the field
 // scratch.
 template <typename T>
@@ -349,16 +368,16 @@ void host_to_field(const klb_lattice *L, const double *drho, const double *u, T 
         host_parallel(nr, nr * nx * 4 * sizeof(double), [&, s, c, nr, fs](size_t r0, size_t r1) {
             for (int a = 0; a < 4; ++a) {
                 const double *in = a == 0 ? (drho ? drho + s * ncell : nullptr) : (u ? u + (s * 3 + a - 1) * ncell : nullptr);
-                for (size_t r = r0; r < r1; ++r) {
-                    T *o = fs + (a * nr + r) * nxp;
-                    if (!in) {
-                        std::memset((void *)o, 0, nxp * sizeof(T));
-                        continue;
-                    }
-                    const double *q = in + nx * g.rows[c][r];
-                    for (size_t x = 0; x < nx; ++x) o[x] = (T)q[x];
-                    for (size_t x = nx; x < nxp; ++x) o[x] = T(0);
+                T *o = fs + (a * nr + r0) * nxp;
+                if (!in) {
+                    std::memset((void *)o, 0, (r1 - r0) * nxp * sizeof(T));
+                    continue;
                 }
+                const int *cs = g.rows[c].data() + r0;
+                fill_rows(o, r1 - r0, nx, nxp, [=](size_t k, T *o) {
+                    const double *q = in + nx * cs[k];
+                    for (size_t x = 0; x < nx; ++x) o[x] = (T)q[x];
+                });
             }
         });
     }
@@ -374,6 +393,8 @@ void rows_to_box(const klb_lattice *L, int cls, size_t planes, double *box, F ro
     host_parallel(n, n * nx * sizeof(double), [&, cls, ncs, nx, box](size_t i0, size_t i1) {
         const int *row_of = g.row_of_cs[cls].data();
         size_t k = i0 / ncs, cs = i0 - k * ncs;
+        const bool narrow = nx < 32;  // zeroed together first, as in fill_rows
+        if (narrow) std::memset(box + i0 * nx, 0, (i1 - i0) * nx * sizeof(double));
         for (size_t i = i0; i < i1;) {
             double *o = box + i * nx;
             if (row_of[cs] >= 0) {
@@ -384,7 +405,7 @@ void rows_to_box(const klb_lattice *L, int cls, size_t planes, double *box, F ro
                 const size_t most = std::min(ncs - cs, i1 - i);
                 size_t m = 1;
                 while (m < most && row_of[cs + m] < 0) ++m;
-                std::memset(o, 0, m * nx * sizeof(double));
+                if (!narrow) std::memset(o, 0, m * nx * sizeof(double));
                 i += m;
                 cs += m;
             }
@@ -915,11 +936,10 @@ klb_status klb_set_state(klb_lattice *L, const double *gin, const double *U1, co
         auto take = [&](auto *pop) {
             using V = std::decay_t<decltype(*pop)>;
             host_parallel((size_t)Q * nr, (size_t)Q * nr * nx * sizeof(double), [&, pop, nr, s, c](size_t k0, size_t k1) {
-                for (size_t k = k0; k < k1; ++k) {
-                    const size_t i = k / nr, r = k - i * nr;
-                    const double *in = gin + ((size_t)s * Q + i) * ncell + nx * g.rows[c][r];
-                    V *o = pop + k * nxp;
-                    std::memset((void *)(o + nx), 0, (nxp - nx) * sizeof(V));
+                const int *cs = g.rows[c].data();
+                size_t i = k0 / nr, r = k0 - i * nr;
+                fill_rows(pop + k0 * nxp, k1 - k0, nx, nxp, [&](size_t, V *o) {
+                    const double *in = gin + ((size_t)s * Q + i) * ncell + nx * cs[r];
                     if constexpr (std::is_same_v<V, __half> || std::is_same_v<V, __nv_bfloat16>) {
                         // Reference of each (row, direction): the x-average of the state.
                         double sum = 0.0;
@@ -936,7 +956,11 @@ klb_status klb_set_state(klb_lattice *L, const double *gin, const double *U1, co
                     } else {
                         for (size_t x = 0; x < nx; ++x) o[x] = (V)in[x];
                     }
-                }
+                    if (++r == nr) {
+                        r = 0;
+                        ++i;
+                    }
+                });
             });
         };
         char *pop = pops.p.get() + (p.pop[0][s] - p.pop[0][0]);
@@ -983,13 +1007,11 @@ klb_status klb_set_state(klb_lattice *L, const double *gin, const double *U1, co
                 using V = std::decay_t<decltype(*U)>;
                 const size_t na = c == kFluid ? 3 : 6, b0 = c == kFluid ? 0 : 3;  // component planes, first box plane
                 host_parallel(na * ns, na * ns * nx * sizeof(double), [&, U, ns, b0, c, t](size_t k0, size_t k1) {
-                    for (size_t k = k0; k < k1; ++k) {
-                        const size_t a = k / ns, q = k - a * ns;
+                    fill_rows(U + k0 * nxp, k1 - k0, nx, nxp, [&](size_t k, V *o) {
+                        const size_t a = (k0 + k) / ns, q = k0 + k - a * ns;
                         const double *in = Ui[t] + (b0 + a) * ncell + nx * g.rows[c][g.slot_row[c][q]];
-                        V *o = U + k * nxp;
                         for (size_t x = 0; x < nx; ++x) o[x] = (V)in[x];
-                        for (size_t x = nx; x < nxp; ++x) o[x] = V(0);
-                    }
+                    });
                 });
             };
             char *U = Us[t].p.get() + (at[c] - at[0]);
