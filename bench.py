@@ -503,6 +503,7 @@ def run_sweep(args):
     if rank != 0:
         return
     updates = sites * SWEEP_STEPS * args.steps * world
+    groups, warps = -(-len(lats) // 36), batch.blocks * batch.width // 32
     peak, peak_kind = _peaks()
     achieved = bytes_per_launch / (step_ms * 1e-3) / 1e9
     line = {
@@ -522,8 +523,9 @@ def run_sweep(args):
                      "bytes_per_launch": bytes_per_launch, "launch_ms": step_ms},
         "e2e": {"value": updates / (e2e_ms * 1e-3) / 1e6, "unit": "MLUPS",
                 "h2d_bytes_per_step": 40 * len(lats), "d2h_bytes_per_step": 120 * len(lats)},
-        # batched steps (36 lattices per launch), one observation (two kernels) and the reference refreshes per lattice
-        "gpu_launches": args.steps * (SWEEP_STEPS * -(-len(lats) // 36) + 2 * len(lats) +
+        # batched steps (36 lattices per launch where that fills the chip, 8000 warps, else one launch), one
+        # observation (two kernels) and the reference refreshes per lattice
+        "gpu_launches": args.steps * (SWEEP_STEPS * (groups if warps >= 8000 * groups else 1) + 2 * len(lats) +
                                       (2 * len(lats) * SWEEP_STEPS // 32 if storage != "fp32" else 0)),
         "clocks": clk.summary(),
         "observables": {"flow_rate_first3": [o["flow_rate"] for o in obs[:3]],

@@ -329,23 +329,26 @@ klb_status klb_set_state(klb_lattice *lat, const double *g, const double *U1,
 /*
  * Batches (no counterpart in the paper; they serve design sweeps in the
  * shape of the nanotube study of Sec. 5.1): many independent lattices
- * stepped together, one kernel launch per lattice step for all of them
- * (channels of different sizes and parameters).  All members share the lattice kind, the storage
+ * stepped together (channels of different sizes and parameters), one kernel
+ * launch per lattice step for up to 36 of them, or for all of more (several
+ * launches, where each fills the chip).  All members share the lattice kind, the storage
  * type and the CUDA stream; they may stand at different time levels (a
  * request admitted while others run).  A member's step pattern (state buffer
  * parity, lagged-velocity ring slot and, for 16-bit storage, reference
  * generation and refresh) repeats after 6 steps, or 384 with 16-bit storage,
  * so one table of per-lattice kernel arguments per phase of that period
- * describes every step.  The
- * tables live in the caller's device buffer (klb_batch_bytes), with a count
- * of the periods completed since they were built (the step number each
+ * describes every step.  The tables are on the host (350 to 400 bytes per
+ * phase and lattice) and go with the launches; the caller's device buffer
+ * (klb_batch_bytes) holds a copy for batches of more than 36 lattices, and a
+ * count of the periods completed since they were built (the step number each
  * replayed step needs: FP32 storage draws the dither of its fix-up from the
- * cell and the step); a whole period is captured once in a CUDA graph and
- * replayed.  The batch enqueues
+ * cell and the step).  A whole period is captured once in a CUDA graph (28 KB
+ * of arguments per launch) and replayed.  The batch enqueues
  * its work on a stream of its own, ordered after and before the members'
  * stream with events.  Members stay usable on their own between batch calls
  * (observables, fields, state, couplings): the next batch step goes on from a
- * state or couplings replaced in between.  Stepping a member alone takes it
+ * state or couplings replaced in between.  Thermal fluctuations that a member
+ * is given later act on its own steps only.  Stepping a member alone takes it
  * out of phase and the next batch call fails with KLB_ESTATE.
  */
 typedef struct klb_batch klb_batch;

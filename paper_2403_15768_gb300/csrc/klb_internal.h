@@ -24,7 +24,8 @@ constexpr int kRowAlign = 32;
 // Water lives on fluid rows; electrons and phonons share the solid rows.
 enum RowClass { kFluid = 0, kSolid = 1 };
 
-// Per-row table, read once per block (all threads of a block share a row).
+// Per-row table: a warp's threads share a row (with FP64 and in the field and
+// initialisation passes a block's).
 struct RowInfo {
     int32_t src[19];            // (dir' * n_rows + row') * nxp / kRowAlign: first element,
                                 // in kRowAlign units, of the row direction i is pulled from

@@ -1114,8 +1114,8 @@ __global__ void __launch_bounds__(kBlockX, (step_min_blocks<T, S, EP>()))
 // The same with the argument records in the kernel's parameters (constant
 // bank): the step body's uses of a record, most of them operands of the
 // uniform datapath, then cost no shared-memory loads and no copy and barrier
-// ahead of the work.  12-channel sweep, FP32 475 -> 456 us, FP16 439 -> 408;
-// 16 or 56 records make no difference.
+// ahead of the work.  12-channel sweep, FP32 475 -> 456 us, FP16 439 -> 408
+// (16 records to a launch the same).
 template <typename T>
 struct BatchTable {
     StepArgs<T> a[kBatchParams];
