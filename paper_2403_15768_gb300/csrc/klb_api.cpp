@@ -430,20 +430,16 @@ size_t pops_bytes(const klb_lattice *L)
     return L->plan.pop[0][2] - L->plan.pop[0][0] + L->plan.pop_bytes[2];
 }
 
-// Start from rest: every population, reference and lagged velocity is 0.
+// Start from rest: every population, lagged velocity and reference is 0.  The
+// first two lie one after the other in the lattice's buffer up to the row
+// tables, as do the references of a generation: two fills at most (one per
+// region, 12 or 18, took longer than k_init of a tiny lattice).
 klb_status init_from_rest(klb_lattice *L)
 {
     const MemoryPlan &p = L->plan;
-    for (int b = 0; b < 2; ++b)
-        for (int s = 0; s < 3; ++s) KLB_CUDA(L, cudaMemsetAsync(dev(L, p.pop[b][s]), 0, p.pop_bytes[s], L->stream));
-    for (int t = 0; t < 3; ++t)
-        for (int c = 0; c < 2; ++c)
-            if (p.U_bytes[c]) KLB_CUDA(L, cudaMemsetAsync(dev(L, p.U[t][c]), 0, p.U_bytes[c], L->stream));
+    KLB_CUDA(L, cudaMemsetAsync(dev(L, p.pop[0][0]), 0, p.rows[kFluid] - p.pop[0][0], L->stream));
     if (reduced(L))
-        for (int s = 0; s < 3; ++s) {
-            KLB_CUDA(L, cudaMemsetAsync(dev(L, p.ref_enc[0][s]), 0, p.ref_bytes[s], L->stream));
-            KLB_CUDA(L, cudaMemsetAsync(dev(L, p.ref_dec[0][s]), 0, p.ref_bytes[s], L->stream));
-        }
+        KLB_CUDA(L, cudaMemsetAsync(dev(L, p.ref_enc[0][0]), 0, p.ref_enc[1][0] - p.ref_enc[0][0], L->stream));
     return KLB_OK;
 }
 

@@ -1,7 +1,7 @@
 """The host side of klb_set_state and klb_get_state, over a stand-in for the CUDA runtime (device memory is host
 memory, kernel launches do nothing).  Without host memory for the conversions, each allocation failing in turn:
 KLB_ENOMEM, and the lattice's buffers and step stay as they were.  States of narrow, ragged and full rows come back
-as they went in, 0 where a species has no cell, with zero padding."""
+as they went in, 0 where a species has no cell, with zero padding; a lattice starts from rest."""
 import os
 import subprocess
 
@@ -87,6 +87,11 @@ static int round_trip(int nx, int storage)
     klb_info info;
     NEED(klb_create_lattice(&d, buf, bytes, nullptr, &L) == KLB_OK && klb_lattice_info(&d, &info) == KLB_OK);
     std::vector<double> g(3 * 19 * cells), u(9 * cells), h(g.size(), 9.0), v(u.size(), 9.0), w(u.size(), 9.0);
+    NEED(klb_get_state(L, h.data(), v.data(), w.data()) == KLB_OK);  // from rest, over a buffer of 0x7f
+    for (double x : h) NEED(x == 0.0);
+    for (double x : v) NEED(x == 0.0);
+    for (double x : w) NEED(x == 0.0);
+    h.assign(h.size(), 9.0);
     for (size_t k = 0; k < g.size(); ++k) g[k] = (float)(1e-4 * (double)(k % 97 + 1));
     for (size_t k = 0; k < u.size(); ++k) u[k] = (float)(1e-4 * (double)(k % 89 + 1));
     NEED(klb_set_state(L, g.data(), u.data(), u.data(), 2) == KLB_OK);
