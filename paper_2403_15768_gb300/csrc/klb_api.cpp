@@ -424,10 +424,21 @@ klb_status sync(klb_lattice *L)
 }
 
 // A state buffer's three species lie one after the other in it, as do the two
-// classes of a lagged-velocity slot: each goes in one copy.
-size_t pops_bytes(const klb_lattice *L)
+// classes of a lagged-velocity slot (which goes in one copy).  Up to 1 MB the
+// species go in one copy, beyond one after the other through the same host
+// memory, whose first touch costs more than the copy (128x64x64 FP32: 76 MB
+// in one, 25 in three).
+struct PopsCopy {
+    bool one;
+    size_t bytes;  // of host memory
+};
+
+PopsCopy pops_copy(const klb_lattice *L)
 {
-    return L->plan.pop[0][2] - L->plan.pop[0][0] + L->plan.pop_bytes[2];
+    const MemoryPlan &p = L->plan;
+    const size_t all = p.pop[0][2] - p.pop[0][0] + p.pop_bytes[2];
+    if (all <= (1u << 20)) return {true, all};
+    return {false, std::max(p.pop_bytes[0], std::max(p.pop_bytes[1], p.pop_bytes[2]))};
 }
 
 // Start from rest: every population, lagged velocity and reference is 0.  The
@@ -809,18 +820,23 @@ klb_status klb_get_state(klb_lattice *L, double *gout, double *U1, double *U2)
         HostBuf pops, refs[3];
         StreamGuard guard{L->stream};
         const size_t *at = L->plan.pop[L->st.cur];
-        if (!pops.alloc(pops_bytes(L))) return no_host_memory(L);
-        KLB_CUDA(L, cudaMemcpyAsync(pops.p.get(), dev(L, at[0]), pops.bytes, cudaMemcpyDeviceToHost, L->stream));
+        const PopsCopy pc = pops_copy(L);
+        if (!pops.alloc(pc.bytes)) return no_host_memory(L);
         for (int s = 0; s < 3; ++s) {
             if (!refs[s].alloc(L->plan.ref_bytes[s])) return no_host_memory(L);
             if (red)
                 KLB_CUDA(L, cudaMemcpyAsync(refs[s].p.get(), dev(L, L->plan.ref_enc[L->st.gen_buf[L->st.cur]][s]),
                                             refs[s].bytes, cudaMemcpyDeviceToHost, L->stream));
         }
-        klb_status st = sync(L);
-        guard.done = true;
-        if (st != KLB_OK) return st;
         for (int s = 0; s < 3; ++s) {
+            if (s == 0 || !pc.one) {
+                guard.done = false;
+                KLB_CUDA(L, cudaMemcpyAsync(pops.p.get(), dev(L, at[s]), pc.one ? pc.bytes : L->plan.pop_bytes[s],
+                                            cudaMemcpyDeviceToHost, L->stream));
+                klb_status st = sync(L);
+                guard.done = true;
+                if (st != KLB_OK) return st;
+            }
             const int c = cls_of(s);
             const size_t nr = g.rows[c].size();
             // Population values of a row (reduced storage: the stored
@@ -844,7 +860,7 @@ klb_status klb_get_state(klb_lattice *L, double *gout, double *U1, double *U2)
                     }
                 });
             };
-            const char *pop = pops.p.get() + (at[s] - at[0]);
+            const char *pop = pops.p.get() + (pc.one ? at[s] - at[0] : 0);
             switch (storage) {
             case KLB_FP64:
                 put(reinterpret_cast<const double *>(pop));
@@ -914,7 +930,8 @@ klb_status klb_set_state(klb_lattice *L, const double *gin, const double *U1, co
     HostBuf encs[3], decs[3], pops, Us[2];
     StreamGuard guard{L->stream};
     const MemoryPlan &p = L->plan;
-    bool have = pops.alloc(pops_bytes(L));
+    const PopsCopy pc = pops_copy(L);
+    bool have = pops.alloc(pc.bytes);
     for (int t = 0; t < 2; ++t) have = have && Us[t].alloc(p.U[0][1] - p.U[0][0] + p.U_bytes[kSolid]);
     for (int s = 0; red && s < 3; ++s) have = have && encs[s].alloc(p.ref_bytes[s]) && decs[s].alloc(p.ref_bytes[s]);
     if (!have) return no_host_memory(L);
@@ -959,7 +976,7 @@ klb_status klb_set_state(klb_lattice *L, const double *gin, const double *U1, co
                 });
             });
         };
-        char *pop = pops.p.get() + (p.pop[0][s] - p.pop[0][0]);
+        char *pop = pops.p.get() + (pc.one ? p.pop[0][s] - p.pop[0][0] : 0);
         switch (storage) {
         case KLB_FP64:
             take(reinterpret_cast<double *>(pop));
@@ -974,9 +991,17 @@ klb_status klb_set_state(klb_lattice *L, const double *gin, const double *U1, co
             take(reinterpret_cast<__nv_bfloat16 *>(pop));
             break;
         }
+        if (!pc.one) {
+            KLB_CUDA(L, cudaMemcpyAsync(dev(L, p.pop[0][s]), pop, p.pop_bytes[s], cudaMemcpyHostToDevice, L->stream));
+            KLB_CUDA(L, cudaMemcpyAsync(dev(L, p.pop[1][s]), dev(L, p.pop[0][s]), p.pop_bytes[s],
+                                        cudaMemcpyDeviceToDevice, L->stream));
+            if (s < 2) KLB_CUDA(L, cudaStreamSynchronize(L->stream));  // the next species takes this memory
+        }
     }
-    KLB_CUDA(L, cudaMemcpyAsync(dev(L, p.pop[0][0]), pops.p.get(), pops.bytes, cudaMemcpyHostToDevice, L->stream));
-    KLB_CUDA(L, cudaMemcpyAsync(dev(L, p.pop[1][0]), dev(L, p.pop[0][0]), pops.bytes, cudaMemcpyDeviceToDevice, L->stream));
+    if (pc.one) {
+        KLB_CUDA(L, cudaMemcpyAsync(dev(L, p.pop[0][0]), pops.p.get(), pc.bytes, cudaMemcpyHostToDevice, L->stream));
+        KLB_CUDA(L, cudaMemcpyAsync(dev(L, p.pop[1][0]), dev(L, p.pop[0][0]), pc.bytes, cudaMemcpyDeviceToDevice, L->stream));
+    }
     if (red) {
         for (int s = 0; s < 3; ++s) {
             const int c = cls_of(s);

@@ -1,7 +1,7 @@
 """The host side of klb_set_state and klb_get_state, over a stand-in for the CUDA runtime (device memory is host
 memory, kernel launches do nothing).  Without host memory for the conversions, each allocation failing in turn:
-KLB_ENOMEM, and the lattice's buffers and step stay as they were.  States of narrow, ragged and full rows come back
-as they went in, 0 where a species has no cell, with zero padding; a lattice starts from rest."""
+KLB_ENOMEM, and the lattice's buffers and step stay as they were.  States of narrow, ragged and full rows, whose
+species go in one copy (up to 1 MB) or one by one, come back as they went in, 0 where a species has no cell, with zero padding; a lattice starts from rest."""
 import os
 import subprocess
 
@@ -117,7 +117,7 @@ static int round_trip(int nx, int storage)
 
 int main()
 {
-    for (int nx : {1, 5, 25, 26, 31, 32, 33, 51, 52, 64, 130})
+    for (int nx : {1, 5, 25, 26, 31, 32, 33, 51, 52, 64, 130, 700})
         for (int storage : {KLB_FP64, KLB_FP32})
             if (round_trip(nx, storage)) return 1;
     for (int storage = 0; storage < 4; ++storage) {
