@@ -1,7 +1,8 @@
 """The host side of klb_set_state and klb_get_state, over a stand-in for the CUDA runtime (device memory is host
 memory, kernel launches do nothing).  Without host memory for the conversions, each allocation failing in turn:
 KLB_ENOMEM, and the lattice's buffers and step stay as they were.  States of narrow, ragged and full rows, whose
-species go in one copy (up to 1 MB) or one by one, come back as they went in, 0 where a species has no cell, with zero padding; a lattice starts from rest."""
+species go in one copy (up to 1 MB) or one by one, come back as they went in, 0 where a species has no cell, with
+zero padding; a lattice starts from rest."""
 import os
 import subprocess
 
